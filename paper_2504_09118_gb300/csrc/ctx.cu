@@ -683,14 +683,14 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
     // scales for 16-bit storage: s_c = 2^(8 - ceil(log2 max|F_c|))
     if (c->storage != FDTD_F32) {
         CK(c, cudaMemsetAsync(c->d_max, 0, sizeof(unsigned) * 6, c->stream));
-        for (int q = 0; q < 6; ++q) {
-            const float *src = f[q];
-            if (!on_device) {
+        if (on_device)
+            CK(c, launch_maxabs(f, 0, 6, c->nx, c->ny, c->nz, c->d_max, c->stream));
+        else
+            for (int q = 0; q < 6; ++q) {
                 CK(c, cudaMemcpyAsync(c->d_stage, f[q], n * 4, cudaMemcpyHostToDevice, c->stream));
-                src = c->d_stage;
+                const float *src = c->d_stage;
+                CK(c, launch_maxabs(&src, q, 1, c->nx, c->ny, c->nz, c->d_max, c->stream));
             }
-            CK(c, launch_maxabs(src, q, c->nx, c->ny, c->nz, c->d_max + q, c->stream));
-        }
         unsigned hm[6];
         CK(c, cudaMemcpyAsync(hm, c->d_max, sizeof hm, cudaMemcpyDeviceToHost, c->stream));
         CK(c, cudaStreamSynchronize(c->stream));
@@ -735,8 +735,7 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
     if (int rc = upload_desc(c)) return rc;
     CavityDesc d = make_desc(c, 0);
     if (on_device) {
-        for (int q = 0; q < 6; ++q)
-            CK(c, launch_pack(c->storage, d, 0, q, f[q], q >= 3 ? c->face[q - 3] : nullptr, c->stream));
+        CK(c, launch_pack(c->storage, d, 0, 0, 6, f, c->stream));
     } else {
         // host fields: field q is copied into staging buffer q & 1 on the copy stream while the
         // previous field is packed on the context's stream (the copy waits until buffer q & 1 is free)
@@ -750,7 +749,8 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
             CK(c, cudaMemcpyAsync(stage, f[q], n * 4, cudaMemcpyHostToDevice, c->copy_stream));
             CK(c, cudaEventRecord(c->staged[b], c->copy_stream));
             CK(c, cudaStreamWaitEvent(c->stream, c->staged[b], 0));
-            CK(c, launch_pack(c->storage, d, 0, q, stage, q >= 3 ? c->face[q - 3] : nullptr, c->stream));
+            const float *src = stage;
+            CK(c, launch_pack(c->storage, d, 0, q, 1, &src, c->stream));
             CK(c, cudaEventRecord(c->packed[b], c->stream));
         }
     }
@@ -815,11 +815,13 @@ int fdtd_get_fields(fdtd_ctx *c, float *const f[6], int on_device) {
     if (!on_device)
         if (int rc = ensure_stage(c)) return rc;
     CavityDesc d = make_desc(c, 0);
-    for (int q = 0; q < 6; ++q) {
-        float *dst = on_device ? f[q] : c->d_stage;
-        CK(c, launch_unpack(c->storage, d, c->cur, q, dst, c->stream));
-        if (!on_device) CK(c, cudaMemcpyAsync(f[q], c->d_stage, n * 4, cudaMemcpyDeviceToHost, c->stream));
-    }
+    if (on_device)
+        CK(c, launch_unpack(c->storage, d, c->cur, 0, 6, f, c->stream));
+    else
+        for (int q = 0; q < 6; ++q) {
+            CK(c, launch_unpack(c->storage, d, c->cur, q, 1, &c->d_stage, c->stream));
+            CK(c, cudaMemcpyAsync(f[q], c->d_stage, n * 4, cudaMemcpyDeviceToHost, c->stream));
+        }
     CK(c, cudaStreamSynchronize(c->stream));
     return check_status(c, c->d_status, c->stream);
 }

@@ -5,6 +5,8 @@
 // then curl E components), each updating one copy of the fields in place; it
 // is the debugging baseline of the fused kernel and the path for coefficient
 // sets too varied for a one-byte material id (COEF_FULL).
+#include <algorithm>
+
 #include "df.cuh"
 #include "launch.h"
 
@@ -14,70 +16,154 @@ namespace {
 
 constexpr int BXs = 32, BYs = 8;
 
-__device__ __forceinline__ bool tangential(int comp, int i, int j, int k) {
-    return (comp == 0 && (j == 0 || k == 0)) || (comp == 1 && (i == 0 || k == 0)) ||
-           (comp == 2 && (i == 0 || j == 0));
+// Up to six canonical arrays of one launch (read by pack and maxabs, written by unpack).
+struct Canon6 {
+    float *f[6];
+};
+
+// Layout conversion.  A warp takes one canonical row (component, k, j), its lanes step along x: the row's
+// kind (cells, or one of the far faces) is the same for the whole warp, the active-layout side is 128-byte
+// aligned, and kLayU loads per lane are issued before their stores.  16-bit rows move two cells per lane, so
+// that a warp still writes (reads) 128 bytes of the active layout at a time.  One launch takes ncomp
+// components: six launches per load cost a small cavity more than the copying did.  Bound by HBM; with
+// one thread per (i, j) and four planes per thread (no row knowledge, single 16-bit stores) the six
+// components took 600 us to load and 834 us to read back at 384^3 FP16, now 358 us (5.7 TB/s) and
+// 476 us; at 256^3 FP32 192 and 166 us, now 144 and 148 us.  Threads over the flat (j, i) index measured
+// 817 and 948 us (stores straddle rows).
+constexpr int kLayThreads = 256, kLayU = 4;
+
+struct LayoutRow {
+    int q, comp, j, k;     // slot in Canon6, component, row
+    bool ok;
+};
+__device__ __forceinline__ LayoutRow layout_row(const CavityDesc &d, int comp0, int ncomp) {
+    LayoutRow r;
+    const unsigned w = blockIdx.x * (kLayThreads / 32) + (threadIdx.x >> 5);
+    const unsigned NY1 = d.ny + 1, NZ1 = d.nz + 1;
+    const unsigned kq = w / NY1;
+    r.j = (int)(w - kq * NY1);
+    r.q = (int)(kq / NZ1);
+    r.k = (int)(kq - (unsigned)r.q * NZ1);
+    r.comp = comp0 + r.q;
+    r.ok = r.q < ncomp;
+    return r;
 }
 
-// Planes per thread of the layout kernels: their loads are issued together before the stores, so that a
-// thread keeps several DRAM reads in flight (one element per thread left these kernels latency-bound).
-constexpr int KZs = 4;
+template <typename T> struct LayPack;   // cells per lane and the store / load of them
+template <> struct LayPack<float> {
+    static constexpr int V = 1;
+    __device__ __forceinline__ static void st(float *p, const float *v) { *p = v[0]; }
+    __device__ __forceinline__ static void ld(const float *p, float *v) { v[0] = *p; }
+};
+template <> struct LayPack<__half> {
+    static constexpr int V = 2;
+    __device__ __forceinline__ static void st(__half *p, const float *v) {
+        *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v[0], v[1]);
+    }
+    __device__ __forceinline__ static void ld(const __half *p, float *v) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(p));
+        v[0] = f.x;
+        v[1] = f.y;
+    }
+};
+template <> struct LayPack<__nv_bfloat16> {
+    static constexpr int V = 2;
+    __device__ __forceinline__ static void st(__nv_bfloat16 *p, const float *v) {
+        *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(v[0], v[1]);
+    }
+    __device__ __forceinline__ static void ld(const __nv_bfloat16 *p, float *v) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+        v[0] = f.x;
+        v[1] = f.y;
+    }
+};
 
+// Value of a far-face H entry after the storage rounding.
+template <typename T> __device__ __forceinline__ float face_round(const CavityDesc &d, int comp, float v) {
+    return Storage<T>::scaled ? Storage<T>::load(Storage<T>::store(v * d.scale[comp])) * d.inv_scale[comp] : v;
+}
+
+// Canonical components -> active layout (scaled, rounded; tangential E zeroed) and far faces.  Rows are
+// padded to a pitch of 32 elements, so a pair that starts inside a row never leaves it; the cell past an odd
+// nx is written 0, as the context's first clear left it.
 template <typename T>
-__device__ __forceinline__ void pack_one(const CavityDesc &d, int copy, int comp, float v, int i, int j, int k,
-                                         float *face) {
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
-    if (i < nx && j < ny && k < nz) {
-        if (comp < 3 && tangential(comp, i, j, k)) v = 0.f;
-        st_field<T>(d, copy, comp, (long long)k * d.plane + (long long)j * d.pitch + i, v);
+__global__ void __launch_bounds__(kLayThreads) pack_kernel(const CavityDesc d, int copy, int comp0, int ncomp,
+                                                           const Canon6 canon) {
+    constexpr int V = LayPack<T>::V;
+    const LayoutRow r = layout_row(d, comp0, ncomp);
+    if (!r.ok) return;
+    const int nx = d.nx, ny = d.ny, nz = d.nz, lane = threadIdx.x & 31;
+    const float *__restrict__ src = canon.f[r.q] + ((long long)r.k * (ny + 1) + r.j) * (nx + 1);
+    float *face = r.comp >= 3 ? const_cast<float *>(d.face[r.comp - 3]) : nullptr;
+    if (r.j < ny && r.k < nz) {
+        T *dst = static_cast<T *>(d.buf[copy][r.comp]) + (long long)r.k * d.plane + (long long)r.j * d.pitch;
+        // Ex is tangential on j = 0 and k = 0, Ey on i = 0 and k = 0, Ez on i = 0 and j = 0
+        const bool zero_row = r.comp < 3 && ((r.k == 0 && r.comp != 2) || (r.j == 0 && r.comp != 1));
+        const bool zero_i0 = r.comp == 1 || r.comp == 2;
+        const float sc = d.scale[r.comp];
+        for (int i0 = lane * V; i0 < nx; i0 += 32 * V * kLayU) {
+            float v[kLayU][V];
+#pragma unroll
+            for (int u = 0; u < kLayU; ++u)
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    const int i = i0 + 32 * V * u + e;
+                    v[u][e] = i < nx && !zero_row && !(zero_i0 && i == 0) ? src[i] : 0.f;
+                }
+#pragma unroll
+            for (int u = 0; u < kLayU; ++u) {
+                const int i = i0 + 32 * V * u;
+                if (Storage<T>::scaled)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) v[u][e] *= sc;
+                if (i < nx) LayPack<T>::st(dst + i, v[u]);
+            }
+        }
+        if (r.comp == 3 && lane == 0) face[(long long)r.k * ny + r.j] = face_round<T>(d, 3, src[nx]);
         return;
     }
-    // far-face normal H: store the value after the same storage rounding
-    float q = v;
-    if (Storage<T>::scaled) q = Storage<T>::load(Storage<T>::store(v * d.scale[comp])) * d.inv_scale[comp];
-    if (comp == 3 && i == nx && j < ny && k < nz) face[(long long)k * ny + j] = q;
-    if (comp == 4 && j == ny && i < nx && k < nz) face[(long long)k * nx + i] = q;
-    if (comp == 5 && k == nz && i < nx && j < ny) face[(long long)j * nx + i] = q;
+    // far-face normal H (FP32, after the same storage rounding)
+    if (r.comp == 4 && r.j == ny && r.k < nz)
+        for (int i = lane; i < nx; i += 32) face[(long long)r.k * nx + i] = face_round<T>(d, 4, src[i]);
+    if (r.comp == 5 && r.k == nz && r.j < ny)
+        for (int i = lane; i < nx; i += 32) face[(long long)r.j * nx + i] = face_round<T>(d, 5, src[i]);
 }
 
-// Canonical component -> active layout (and far faces); each thread takes KZs planes of one (i, j).
+// Active layout (and far faces) -> canonical components, zero outside the extents.
 template <typename T>
-__global__ void pack_kernel(const CavityDesc d, int copy, int comp, const float *__restrict__ canon, float *face) {
-    const int i = blockIdx.x * BXs + threadIdx.x, j = blockIdx.y * BYs + threadIdx.y, k0 = blockIdx.z * KZs;
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
-    if (i > nx || j > ny) return;
-    const long long zs = (long long)(ny + 1) * (nx + 1), base = (long long)j * (nx + 1) + i;
-    float v[KZs];
+__global__ void __launch_bounds__(kLayThreads) unpack_kernel(const CavityDesc d, int copy, int comp0, int ncomp,
+                                                             const Canon6 canon) {
+    constexpr int V = LayPack<T>::V;
+    const LayoutRow r = layout_row(d, comp0, ncomp);
+    if (!r.ok) return;
+    const int nx = d.nx, ny = d.ny, nz = d.nz, lane = threadIdx.x & 31;
+    float *__restrict__ dst = canon.f[r.q] + ((long long)r.k * (ny + 1) + r.j) * (nx + 1);
+    if (r.j < ny && r.k < nz) {
+        const T *__restrict__ src =
+            static_cast<const T *>(d.buf[copy][r.comp]) + (long long)r.k * d.plane + (long long)r.j * d.pitch;
+        const float is = d.inv_scale[r.comp];
+        for (int i0 = lane * V; i0 < nx; i0 += 32 * V * kLayU) {
+            float v[kLayU][V];
 #pragma unroll
-    for (int q = 0; q < KZs; ++q) v[q] = k0 + q <= nz ? canon[(k0 + q) * zs + base] : 0.f;
+            for (int u = 0; u < kLayU; ++u) {
+                const int i = i0 + 32 * V * u;
+                if (i < nx) LayPack<T>::ld(src + i, v[u]);
+            }
 #pragma unroll
-    for (int q = 0; q < KZs; ++q)
-        if (k0 + q <= nz) pack_one<T>(d, copy, comp, v[q], i, j, k0 + q, face);
-}
-
-template <typename T>
-__device__ __forceinline__ float unpack_one(const CavityDesc &d, int copy, int comp, int i, int j, int k) {
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
-    if (i < nx && j < ny && k < nz) return ld_field<T>(d, copy, comp, (long long)k * d.plane + (long long)j * d.pitch + i);
-    if (comp == 3 && i == nx && j < ny && k < nz) return d.face[0][(long long)k * ny + j];
-    if (comp == 4 && j == ny && i < nx && k < nz) return d.face[1][(long long)k * nx + i];
-    if (comp == 5 && k == nz && i < nx && j < ny) return d.face[2][(long long)j * nx + i];
-    return 0.f;
-}
-
-// Active layout (and far faces) -> canonical component, zero outside the extent; KZs planes per thread.
-template <typename T>
-__global__ void unpack_kernel(const CavityDesc d, int copy, int comp, float *__restrict__ canon) {
-    const int i = blockIdx.x * BXs + threadIdx.x, j = blockIdx.y * BYs + threadIdx.y, k0 = blockIdx.z * KZs;
-    const int nx = d.nx, ny = d.ny, nz = d.nz;
-    if (i > nx || j > ny) return;
-    const long long zs = (long long)(ny + 1) * (nx + 1), base = (long long)j * (nx + 1) + i;
-    float v[KZs];
+            for (int u = 0; u < kLayU; ++u)
 #pragma unroll
-    for (int q = 0; q < KZs; ++q) v[q] = k0 + q <= nz ? unpack_one<T>(d, copy, comp, i, j, k0 + q) : 0.f;
-#pragma unroll
-    for (int q = 0; q < KZs; ++q)
-        if (k0 + q <= nz) canon[(k0 + q) * zs + base] = v[q];
+                for (int e = 0; e < V; ++e) {
+                    const int i = i0 + 32 * V * u + e;
+                    if (i < nx) dst[i] = Storage<T>::scaled ? v[u][e] * is : v[u][e];
+                }
+        }
+        if (lane == 0) dst[nx] = r.comp == 3 ? d.face[0][(long long)r.k * ny + r.j] : 0.f;
+        return;
+    }
+    const float *__restrict__ face = nullptr;
+    if (r.comp == 4 && r.j == ny && r.k < nz) face = d.face[1] + (long long)r.k * nx;
+    if (r.comp == 5 && r.k == nz && r.j < ny) face = d.face[2] + (long long)r.j * nx;
+    for (int i = lane; i <= nx; i += 32) dst[i] = face && i < nx ? face[i] : 0.f;
 }
 
 __device__ __forceinline__ bool in_extent(int comp, int i, int j, int k, int nx, int ny, int nz) {
@@ -91,13 +177,43 @@ __device__ __forceinline__ bool in_extent(int comp, int i, int j, int k, int nx,
     }
 }
 
-__global__ void maxabs_kernel(const float *__restrict__ canon, int comp, int nx, int ny, int nz, unsigned *out) {
-    const int i = blockIdx.x * BXs + threadIdx.x, j = blockIdx.y * BYs + threadIdx.y, k = blockIdx.z;
-    float v = 0.f;
-    if (i <= nx && j <= ny && in_extent(comp, i, j, k, nx, ny, nz))
-        v = fabsf(canon[((long long)k * (ny + 1) + j) * (nx + 1) + i]);
+// max |canon| over the component's extent into out[component].  A warp takes whole extent rows (so no
+// element needs its own index arithmetic), a lane four loads at a time; a block reduces in shared memory
+// and issues one atomic.  Bound by HBM reads: 331 us for the six 384^3 components (4.1 TB/s).  One atomic
+// per warp, all on one address per component, took 7.6 ms.
+constexpr int kMaxThreads = 256;
+__global__ void __launch_bounds__(kMaxThreads) maxabs_kernel(const Canon6 canon, int comp0, int nx, int ny, int nz,
+                                                             unsigned *out) {
+    __shared__ float sh[kMaxThreads / 32];
+    const int comp = comp0 + blockIdx.y;
+    const float *__restrict__ src = canon.f[blockIdx.y];
+    const int ex = nx + (in_extent(comp, nx, 0, 0, nx, ny, nz) ? 1 : 0);
+    const int ey = ny + (in_extent(comp, 0, ny, 0, nx, ny, nz) ? 1 : 0);
+    const int ez = nz + (in_extent(comp, 0, 0, nz, nx, ny, nz) ? 1 : 0);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long rows = (long long)ey * ez, stride = (long long)gridDim.x * (kMaxThreads / 32);
+    float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
+    for (long long r = (long long)blockIdx.x * (kMaxThreads / 32) + w; r < rows; r += stride) {
+        const long long k = r / ey;
+        const float *row = src + (k * (ny + 1) + (r - k * ey)) * (nx + 1);
+        int i = lane;
+        for (; i + 96 < ex; i += 128) {
+            const float a = row[i], b = row[i + 32], c = row[i + 64], e = row[i + 96];
+            m0 = fmaxf(m0, fabsf(a));
+            m1 = fmaxf(m1, fabsf(b));
+            m2 = fmaxf(m2, fabsf(c));
+            m3 = fmaxf(m3, fabsf(e));
+        }
+        for (; i < ex; i += 32) m0 = fmaxf(m0, fabsf(row[i]));
+    }
+    float v = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));   // fmaxf passes over NaN, as the extent scan always did
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0 && v > 0.f) atomicMax(out, __float_as_uint(v));
+    if (lane == 0) sh[w] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < kMaxThreads / 32; ++q) v = fmaxf(v, sh[q]);
+        if (v > 0.f) atomicMax(out + comp, __float_as_uint(v));
+    }
 }
 
 // H^{n+1/2} = H^{n-1/2} - ch curl E^n, one thread per cell (E beyond the active range is 0).
@@ -326,22 +442,39 @@ cudaError_t simple_step_typed(const CavityDesc &d, int copy, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_pack(int storage, const CavityDesc &d, int copy, int comp, const float *canon, float *face,
+// Device memory bounds ny nz at about 3.6e8 (rows are padded to 32 elements, 12 arrays of them must fit), so row
+// numbers fit 32 bits.
+static unsigned layout_blocks(const CavityDesc &d, int ncomp) {
+    const unsigned long long rows = (unsigned long long)ncomp * (d.ny + 1) * (d.nz + 1);
+    return (unsigned)((rows + kLayThreads / 32 - 1) / (kLayThreads / 32));
+}
+
+cudaError_t launch_pack(int storage, const CavityDesc &d, int copy, int comp0, int ncomp, const float *const *canon,
                         cudaStream_t s) {
-    dim3 blk(BXs, BYs), grd((d.nx + 1 + BXs - 1) / BXs, (d.ny + 1 + BYs - 1) / BYs, (d.nz + 1 + KZs - 1) / KZs);
-    FDTD_STORAGE_DISPATCH(storage, pack_kernel<T><<<grd, blk, 0, s>>>(d, copy, comp, canon, face));
+    Canon6 c{};
+    for (int q = 0; q < ncomp; ++q) c.f[q] = const_cast<float *>(canon[q]);
+    const unsigned grd = layout_blocks(d, ncomp);
+    FDTD_STORAGE_DISPATCH(storage, pack_kernel<T><<<grd, kLayThreads, 0, s>>>(d, copy, comp0, ncomp, c));
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack(int storage, const CavityDesc &d, int copy, int comp, float *canon, cudaStream_t s) {
-    dim3 blk(BXs, BYs), grd((d.nx + 1 + BXs - 1) / BXs, (d.ny + 1 + BYs - 1) / BYs, (d.nz + 1 + KZs - 1) / KZs);
-    FDTD_STORAGE_DISPATCH(storage, unpack_kernel<T><<<grd, blk, 0, s>>>(d, copy, comp, canon));
+cudaError_t launch_unpack(int storage, const CavityDesc &d, int copy, int comp0, int ncomp, float *const *canon,
+                          cudaStream_t s) {
+    Canon6 c{};
+    for (int q = 0; q < ncomp; ++q) c.f[q] = canon[q];
+    const unsigned grd = layout_blocks(d, ncomp);
+    FDTD_STORAGE_DISPATCH(storage, unpack_kernel<T><<<grd, kLayThreads, 0, s>>>(d, copy, comp0, ncomp, c));
     return cudaGetLastError();
 }
 
-cudaError_t launch_maxabs(const float *canon, int comp, int nx, int ny, int nz, unsigned *out, cudaStream_t s) {
-    dim3 blk(BXs, BYs), grd((nx + 1 + BXs - 1) / BXs, (ny + 1 + BYs - 1) / BYs, nz + 1);
-    maxabs_kernel<<<grd, blk, 0, s>>>(canon, comp, nx, ny, nz, out);
+cudaError_t launch_maxabs(const float *const *canon, int comp0, int ncomp, int nx, int ny, int nz, unsigned *out,
+                          cudaStream_t s) {
+    Canon6 c{};
+    for (int q = 0; q < ncomp; ++q) c.f[q] = const_cast<float *>(canon[q]);
+    // enough warps for every row once, at most about eight blocks per SM over the launch's components
+    const long long rows = (long long)(ny + 1) * (nz + 1), per = kMaxThreads / 32;
+    const int blocks = (int)std::min<long long>((rows + per - 1) / per, 1216 / ncomp + 1);
+    maxabs_kernel<<<dim3(blocks, ncomp), kMaxThreads, 0, s>>>(c, comp0, nx, ny, nz, out);
     return cudaGetLastError();
 }
 

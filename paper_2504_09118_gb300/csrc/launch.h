@@ -5,14 +5,16 @@
 
 namespace fdtd {
 
-// Canonical FP32 component -> active array (scaled, rounded to storage), tangential E zeroed,
-// far-face normal H -> face array (FP32, after the same rounding).
-cudaError_t launch_pack(int storage, const CavityDesc &d, int copy, int comp, const float *canon, float *face,
+// Canonical FP32 components comp0 .. comp0 + ncomp - 1 (canon[0 .. ncomp)) -> active arrays (scaled, rounded
+// to storage), tangential E zeroed, far-face normal H -> the face arrays (FP32, after the same rounding).
+cudaError_t launch_pack(int storage, const CavityDesc &d, int copy, int comp0, int ncomp, const float *const *canon,
                         cudaStream_t s);
-// Active array (+ face) -> canonical FP32 component, zero outside the extent.
-cudaError_t launch_unpack(int storage, const CavityDesc &d, int copy, int comp, float *canon, cudaStream_t s);
-// max |canon| over the component's extent, as float bits atomically max-ed into *out (must start at 0).
-cudaError_t launch_maxabs(const float *canon, int comp, int nx, int ny, int nz, unsigned *out, cudaStream_t s);
+// Active arrays (+ faces) -> canonical FP32 components, zero outside the extents.
+cudaError_t launch_unpack(int storage, const CavityDesc &d, int copy, int comp0, int ncomp, float *const *canon,
+                          cudaStream_t s);
+// max |canon[q]| over each component's extent, as float bits atomically max-ed into out[comp0 + q] (0 at start).
+cudaError_t launch_maxabs(const float *const *canon, int comp0, int ncomp, int nx, int ny, int nz, unsigned *out,
+                          cudaStream_t s);
 // One unfused step in place on copy `copy`: H kernel then E kernel.
 cudaError_t launch_simple_step(int storage, const CavityDesc &d, int copy, cudaStream_t s);
 // Reductions accumulated in FP64: what == 0 gives out[0] = sum E^2/ce + H.(H - ch curl E)/ch;
