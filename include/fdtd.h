@@ -72,8 +72,12 @@ enum fdtd_status {
 
 /* Step kernels (fdtd_tuning.kernel). */
 enum fdtd_kernel {
-    FDTD_KERNEL_AUTO = 0,    /* TEMPORAL with 16-row tiles where it applies (else FUSED; SIMPLE for
-                                per-position coefficient arrays); fdtd_autotune picks by timing */
+    FDTD_KERNEL_AUTO = 0,    /* with no launch-shape field set: calls of 4 steps or more on a small second-order
+                                cavity (about 10^6 cells or fewer, at most 31 materials, no slab) keep the state
+                                on chip, many steps per launch (FP32: bit for bit the other kernels' results;
+                                16-bit storage is rounded once per launch).  Else TEMPORAL with 16-row tiles
+                                where it applies (else FUSED; SIMPLE for per-position coefficient arrays);
+                                fdtd_autotune picks among the tiled kernels by timing */
     FDTD_KERNEL_SIMPLE = 1,  /* two launches per step (H, then E), one thread per cell; unfused baseline */
     FDTD_KERNEL_FUSED = 2,   /* one TMA-pipelined launch per step: H then E fused in a z-march */
     FDTD_KERNEL_TEMPORAL = 3, /* two steps per launch (temporal blocking); an odd count ends with one FUSED step */
@@ -247,7 +251,9 @@ FDTD_API int fdtd_autotune(fdtd_ctx *ctx, int trial_steps, fdtd_tuning *out, dou
  * an E position inside the cavity and not tangential to a face (ERR_ARG otherwise).  Sources at the
  * same position add up.  nsrc = 0 removes them.  All arrays are host memory, copied.  While currents
  * or probes are set, steps run the one-step kernel followed by one small launch for them (the
- * two-step kernel has no point between its steps where J could enter).  Synchronises the stream. */
+ * two-step kernel has no point between its steps where J could enter), or, under AUTO on a small cavity
+ * with at most 32 currents and 256 probes, on chip with the currents and probes in the same launch.
+ * Synchronises the stream. */
 FDTD_API int fdtd_set_sources(fdtd_ctx *ctx, int nsrc, const int *comp, const int *ijk, const float *wave,
                               int wave_len);
 

@@ -101,6 +101,11 @@ struct fdtd_ctx {
         int *first = nullptr;   // inside the same allocation as d
         int n = 0, grid = 0, key = 0;
     } tl[4];                                // [0] one-step, [1] two-step, [2] fourth-order, [3] three-step kernel
+    // many steps per launch on chip (k_resident.cu; small cavities under AUTO): boxes per axis and, allocated
+    // with the first such launch, the surface buffers followed by the tag counter
+    int resident = 0;                       // 0: not looked at yet, 1: available, -1: not available
+    int resident_parts[3] = {0, 0, 0};
+    void *d_resident = nullptr;
     int order = 2;                          // spatial order of the differences (2: Eq. 2, 4: the (2,4) scheme)
     double courant = 0.0;                   // max over cells of 3 ce ch (stable for order 2 when <= 1)
     int ch_uniform = 1;
@@ -239,6 +244,7 @@ void slab_took_steps(fdtd_ctx *c, int nsteps);
 
 // ---- point currents and probes (extras_api.cu)
 bool extras_on(const fdtd_ctx *c);
+ExtrasParams make_extras(const fdtd_ctx *c);
 int launch_extras_after(fdtd_ctx *c, int copy);
 
 // ---- autotuning (autotune.cu)

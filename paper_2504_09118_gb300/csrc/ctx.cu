@@ -600,6 +600,7 @@ void fdtd_destroy(fdtd_ctx *c) {
         pool_free(p, st);
     pool_free(c->d_stage2, st);
     pool_free(c->d_prefetch, st);
+    pool_free(c->d_resident, st);
     cudaStreamSynchronize(st);
     if (c->copy_stream) {
         cudaStreamSynchronize(c->copy_stream);
@@ -826,6 +827,88 @@ int fdtd_get_fields(fdtd_ctx *c, float *const f[6], int on_device) {
     return check_status(c, c->d_status, c->stream);
 }
 
+// Steps a resident launch takes at least and at most.  A launch loads and stores the whole state, which a few
+// steps do not repay; the cap keeps a launch near a millisecond, so that another stream's
+// kernels wait no longer than that for the SMs.
+constexpr int kResidentMinSteps = 4, kResidentMaxSteps = 256;
+
+// Whether nsteps steps may run on chip: AUTO with no launch-shape field set, second order, materials or a
+// uniform cavity, few enough cells, currents and probes.
+static bool use_resident(fdtd_ctx *c, int nsteps) {
+    const fdtd_tuning &t = c->tuning;
+    if (c->resident < 0 || nsteps < kResidentMinSteps || c->order != 2 || c->slab.on) return false;
+    if (t.kernel != FDTD_KERNEL_AUTO || t.tile_y || t.zchunk || t.ctas_per_sm || t.stages) return false;
+    if (!(c->coef_mode == COEF_SCALAR || (c->coef_mode == COEF_ID8 && c->id_pec))) return false;
+    if (c->nsrc > kResidentMaxSources || c->nprobe > kResidentMaxProbes) return false;
+    if (c->resident == 0)
+        c->resident = 6 * c->arr_elems < (size_t)INT_MAX && resident_split(c->nx, c->ny, c->nz, num_sms(), c->resident_parts)
+                          ? 1 : -1;
+    return c->resident > 0;
+}
+
+// n steps on chip.  FDTD_OK with *done = false (nothing enqueued) when the device cannot run the launch or there
+// is no room for its buffers: the caller then takes the tiled kernels.
+static int step_resident(fdtd_ctx *c, int n, bool *done) {
+    *done = false;
+    const int *parts = c->resident_parts;
+    const size_t words = resident_word_bytes(c->nz, parts);
+    if (!c->d_resident) {
+        if (dmalloc(c, &c->d_resident, words + 2 * sizeof(unsigned)) != cudaSuccess) {
+            cudaGetLastError();
+            c->d_resident = nullptr;
+            c->resident = -1;
+            return FDTD_OK;
+        }
+        CK(c, cudaMemsetAsync(c->d_resident, 0, words + 2 * sizeof(unsigned), c->stream));
+    }
+    const TileRec r = base_rec(c, 0, 1);   // coefficients in storage units, PEC-coded table
+    ResidentParams P{};
+    P.src = c->fields[c->cur][0];
+    P.dst = c->fields[c->cur ^ 1][0];
+    P.storage = c->storage;
+    P.fstride = (int)c->arr_elems;
+    P.nx = c->nx;
+    P.ny = c->ny;
+    P.nz = c->nz;
+    P.pitch = c->pitch;
+    P.plane = c->pitch * c->ny;
+    P.px = parts[0];
+    P.py = parts[1];
+    P.pz = parts[2];
+    P.steps = n;
+    for (int q = 0; q < 3; ++q) {
+        P.ce[q] = r.ce[q];
+        P.ch[q] = r.ch[q];
+        P.ce_mat[q] = c->ce_s[q];
+    }
+    if (c->coef_mode == COEF_ID8) {
+        P.id = c->id_pec;
+        P.table = r.table;
+        P.ntab = r.ntab;
+        P.id_mat = c->id;
+        P.table_mat = c->table;
+    }
+    P.ch_uniform = c->ch_uniform;
+    P.scale_e = c->scale[0];
+    P.inv_scale_e = 1.0f / c->scale[0];
+    P.inv_scale_h = 1.0f / c->scale[3];
+    P.words = c->d_resident;
+    P.epoch = reinterpret_cast<unsigned *>(static_cast<char *>(c->d_resident) + words);
+    P.status = c->d_status;
+    if (extras_on(c)) P.X = make_extras(c);
+    const cudaError_t e = launch_resident(P, c->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        c->resident = -1;
+        return FDTD_OK;
+    }
+    CK(c, e);
+    c->cur ^= 1;
+    c->steps += n;
+    *done = true;
+    return FDTD_OK;
+}
+
 int fdtd_step(fdtd_ctx *c, int nsteps) {
     NvtxRange nvtx_range("fdtd_step");
     if (!c) return FDTD_ERR_ARG;
@@ -839,6 +922,17 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
     // currents enter between the E update of one step and the H update of the next: one step per launch
     const bool temporal = use_temporal(c) && !extras;
     const int k1 = one_step_kind(c);
+    int left = nsteps;
+    if (c->inject_us <= 0)
+        while (use_resident(c, left)) {
+            const int launches = (left + kResidentMaxSteps - 1) / kResidentMaxSteps;
+            const int n = (left + launches - 1) / launches;   // equal shares: no short last launch
+            bool done = false;
+            if (int rc = step_resident(c, n, &done)) return rc;
+            if (!done) break;
+            left -= n;
+        }
+    if (left == 0) return FDTD_OK;
     if (fused)
         if (int rc = build_tiles(c, k1)) return rc;
     // kind 1 (two steps per launch) or 3 (three steps per launch)
@@ -851,7 +945,6 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
         if (int rc = launch_one(c, parity, inj, kind)) return rc;
         return extras ? launch_extras_after(c, fused ? parity ^ 1 : c->cur) : FDTD_OK;
     };
-    int left = nsteps;
     if (c->inject_us > 0 && fused) {
         const int inj = c->inject_us;
         c->inject_us = 0;

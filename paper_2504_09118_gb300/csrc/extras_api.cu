@@ -6,8 +6,7 @@ namespace fdtd {
 
 bool extras_on(const fdtd_ctx *c) { return c->nsrc > 0 || c->nprobe > 0; }
 
-// The point-current / probe launch after a step that left the state in copy `copy`.
-int launch_extras_after(fdtd_ctx *c, int copy) {
+ExtrasParams make_extras(const fdtd_ctx *c) {
     ExtrasParams X{};
     X.clock = c->d_xclock;
     X.nsrc = c->nsrc;
@@ -22,7 +21,12 @@ int launch_extras_after(fdtd_ctx *c, int copy) {
     X.probe_comp = c->d_probe_comp;
     X.probe_off = c->d_probe_off;
     X.probe_buf = c->d_probe_buf;
-    CK(c, launch_extras(c->storage, make_desc(c, 0), copy, X, c->stream));
+    return X;
+}
+
+// The point-current / probe launch after a step that left the state in copy `copy`.
+int launch_extras_after(fdtd_ctx *c, int copy) {
+    CK(c, launch_extras(c->storage, make_desc(c, 0), copy, make_extras(c), c->stream));
     return FDTD_OK;
 }
 

@@ -84,6 +84,34 @@ struct ExtrasParams {
 };
 cudaError_t launch_extras(int storage, const CavityDesc &d, int copy, const ExtrasParams &X, cudaStream_t s);
 
+// Many steps of a small cavity in one cooperative launch, the state on chip (k_resident.cu).
+constexpr int kResidentMaxBZ = 14;       // cells per box along z (at most 32 along x, 16 along y)
+constexpr int kResidentMaxSources = 32, kResidentMaxProbes = 256;
+struct ResidentParams {
+    const void *src;           // first of the six source arrays, fstride elements apart
+    void *dst;                 // first of the six result arrays
+    int storage;
+    int fstride;
+    int nx, ny, nz, pitch, plane;
+    int px, py, pz;            // boxes along each axis
+    int steps;
+    float ce[3], ch[3];        // in storage units (TileRec); ch also when ch_uniform
+    const uint8_t *id;         // PEC-coded ids (NULL: uniform cavity) and their table, ntab entries
+    const float4 *table;
+    int ntab, ch_uniform;
+    float scale_e, inv_scale_e, inv_scale_h;
+    float ce_mat[3];           // unscaled coefficients for currents: scalars, or table by plain id
+    const uint8_t *id_mat;
+    const float *table_mat;
+    void *words;               // surface buffers of every box, two copies (resident_word_bytes, zero at first)
+    unsigned *epoch;           // step tag the next launch starts from, and a count of CTAs (both 0 at first)
+    int *status;
+    ExtrasParams X;            // currents and probes (nsrc = nprobe = 0: none); advances X.clock
+};
+bool resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]);
+size_t resident_word_bytes(int nz, const int parts[3]);
+cudaError_t launch_resident(const ResidentParams &P, cudaStream_t s);
+
 // Adds inc to the device step clock of a batch (one thread; ordered after the launch it follows).
 cudaError_t launch_step_counter(long long *counter, int inc, cudaStream_t s);
 // Two-step (temporal blocking) kernel: output tile width along x, shared memory, occupancy, launch.
