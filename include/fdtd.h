@@ -75,12 +75,15 @@ enum fdtd_kernel {
     FDTD_KERNEL_AUTO = 0,    /* with no launch-shape field set: calls of 4 steps or more on a small second-order
                                 cavity (about 10^6 cells or fewer, at most 31 materials, no slab) keep the state
                                 on chip, many steps per launch (FP32: bit for bit the other kernels' results;
-                                16-bit storage is rounded once per launch).  Else TEMPORAL with 16-row tiles
-                                where it applies (else FUSED; SIMPLE for per-position coefficient arrays);
-                                fdtd_autotune picks among the tiled kernels by timing */
+                                16-bit storage is rounded once per launch).  Else TEMPORAL where it applies
+                                (second order, per-position coefficient arrays included), else FUSED, else
+                                SIMPLE (fourth order with per-position coefficient arrays); fdtd_autotune picks
+                                among the tiled kernels by timing */
     FDTD_KERNEL_SIMPLE = 1,  /* two launches per step (H, then E), one thread per cell; unfused baseline */
     FDTD_KERNEL_FUSED = 2,   /* one TMA-pipelined launch per step: H then E fused in a z-march */
-    FDTD_KERNEL_TEMPORAL = 3, /* two steps per launch (temporal blocking); an odd count ends with one FUSED step */
+    FDTD_KERNEL_TEMPORAL = 3, /* two steps per launch (temporal blocking); an odd count ends with one FUSED step.
+                                 Per-position coefficient arrays: 12-row tiles that stream the arrays with the
+                                 fields, an odd count ends with one SIMPLE step */
     FDTD_KERNEL_TEMPORAL2 = 4, /* TEMPORAL with two tile rows per consumer warp (tile_y 12 or 16): same tiles and
                                  results (FP32: bit for bit), fewer instructions per cell-step */
     FDTD_KERNEL_TEMPORAL3 = 5 /* three steps per launch (single cavities, second order; tile_y 8, 10 or 12; 58-column
@@ -237,7 +240,8 @@ FDTD_API int fdtd_get_order(const fdtd_ctx *ctx);
  * of the active arrays, freed before return) and restored afterwards, so the state and
  * fdtd_steps_done are unchanged.  The choice is kept per (nx, ny, nz, storage, coefficient
  * kind, spatial order) for the life of the process: a later call for the same shape applies it
- * without trials.  Contexts with per-position coefficient arrays keep the unfused kernel; with
+ * without trials.  Contexts with per-position coefficient arrays are not timed and get SIMPLE (AUTO's
+ * two-step kernel is faster on them: do not autotune those); with
  * order 4 the candidates are the fused fourth-order kernel with 4, 8, 12, 16-row tiles and the
  * deepest ring that fits or 4 slots.  out
  * (may be NULL) receives the chosen tuning, ms_per_step (may be NULL) its time per step.

@@ -75,7 +75,7 @@ struct fdtd_ctx {
     uint8_t *id_pec = nullptr;
     float *table_pec = nullptr;
     int ntab_pec = 0;
-    float *coef_full[6] = {};
+    float *coef_full[6] = {};         // one allocation, arr_elems apart
     float scale[6] = {1, 1, 1, 1, 1, 1};
     int cur = 0;
     long long steps = 0;
@@ -94,13 +94,14 @@ struct fdtd_ctx {
     unsigned *d_max = nullptr;
     CUtensorMap *d_maps = nullptr;          // kMapSets x kMapsPerCavity
     std::vector<CUtensorMap> host_maps[kMapSets];
-    int maps_by[kMapSets] = {0, 0, 0, 0};   // box height each map set was encoded for (0: not yet)
+    int maps_by[kMapSets] = {};   // box height each map set was encoded for (0: not yet)
     CavityDesc *d_desc = nullptr;
     struct TileList {
         TileRec *d = nullptr;   // records, followed by the per-CTA range offsets
         int *first = nullptr;   // inside the same allocation as d
         int n = 0, grid = 0, key = 0;
-    } tl[4];                                // [0] one-step, [1] two-step, [2] fourth-order, [3] three-step kernel
+    } tl[5];                                // [0] one-step, [1] two-step, [2] fourth-order, [3] three-step kernel,
+                                            // [4] two-step kernel with per-position coefficients
     // many steps per launch on chip (k_resident.cu; small cavities under AUTO): boxes per axis and, allocated
     // with the first such launch, the surface buffers followed by the tag counter
     int resident = 0;                       // 0: not looked at yet, 1: available, -1: not available
@@ -211,6 +212,7 @@ int encode_maps(fdtd_ctx *c, int set, int box_y);
 void drop_graphs(std::map<GraphKey, cudaGraphExec_t> &g);
 bool use_fused(const fdtd_ctx *c);
 bool use_temporal(const fdtd_ctx *c);
+bool use_full2(const fdtd_ctx *c);
 int one_step_kind(const fdtd_ctx *c);
 int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind = 0);
 int check_status(fdtd_ctx *c, int *d_status, cudaStream_t s);
@@ -219,13 +221,14 @@ int ensure_stage2(fdtd_ctx *c);
 
 // ---- launch planning (plan.cu)
 struct Shape {
-    int kind;   // 0: one step per launch, 1: two steps per launch, 2: one fourth-order step, 3: three steps
+    int kind;   // 0: one step per launch, 1: two steps per launch, 2: one fourth-order step, 3: three steps,
+                // 4: two steps per launch with per-position coefficients
     int tile_y, stages, ctas_per_sm;
     int rows_per_warp;   // kind 1: rows per consumer warp (1, or 2 for FDTD_KERNEL_TEMPORAL2)
 };
 // Rows per consumer warp of the two-step kernel a tuning selects.
 inline int two_step_rows(const fdtd_tuning &t) { return t.kernel == FDTD_KERNEL_TEMPORAL2 ? 2 : 1; }
-Shape resolve_shape(int storage, const fdtd_tuning &t, int kind = 0);
+Shape resolve_shape(int storage, const fdtd_tuning &t, int kind = 0, bool full_ch = false);
 int choose_zlen(long long cols, int nz, int grid, int zchunk, int prologue_planes);
 long long simulate_plan(const std::vector<int> &plan, long long cols, int G, int prologue);
 std::vector<int> plan_chunks(long long cols, int nz, int G, int prologue, int zchunk);

@@ -101,7 +101,7 @@ int encode_maps(fdtd_ctx *c, int set, int box_y) {
     // field box width: one granule of halo on each side of the 64 lane cells, except for the two- and
     // three-step kernels, whose lane cells start left of the tile and whose box origin is rounded down to
     // the granule: 64 + one granule
-    const int bx = (set == 1 || set == 3) ? kTileX + hx : kTileX + 2 * hx;
+    const int bx = (set == 1 || set == 3 || set == 4) ? kTileX + hx : kTileX + 2 * hx;
     std::vector<CUtensorMap> &maps = c->host_maps[set];
     maps.assign(kMapsPerCavity, CUtensorMap{});
     const size_t es = esize(c->storage);
@@ -131,6 +131,16 @@ int encode_maps(fdtd_ctx *c, int set, int box_y) {
                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return fail(c, FDTD_ERR_CUDA, "4-D tensor map encode failed (%d)", (int)r);
         }
+    if (set == 4) {   // per-position coefficients: one 4-D FP32 map over the ce (and ch) arrays
+        cuuint64_t gdim4[4] = {(cuuint64_t)c->nx, (cuuint64_t)c->ny, (cuuint64_t)c->nz, 6};
+        cuuint64_t gstr4[3] = {(cuuint64_t)c->pitch * 4, (cuuint64_t)c->pitch * c->ny * 4, (cuuint64_t)c->arr_elems * 4};
+        cuuint32_t box4[4] = {(cuuint32_t)(kTileX + 4), (cuuint32_t)box_y, 1, (cuuint32_t)(c->ch_uniform ? 3 : 6)};
+        cuuint32_t estr4[4] = {1, 1, 1, 1};
+        CUresult r = enc(&maps[12], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->coef_full[0], gdim4, gstr4, box4, estr4,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return fail(c, FDTD_ERR_CUDA, "coefficient tensor map encode failed (%d)", (int)r);
+    }
     if (c->id) {
         cuuint64_t gstr[2] = {(cuuint64_t)c->pitch, (cuuint64_t)c->pitch * c->ny};
         // ids from 16 bytes left of the tile; the fourth-order kernel also needs its right halo
@@ -167,22 +177,29 @@ bool use_temporal(const fdtd_ctx *c) {
             c->tuning.kernel == FDTD_KERNEL_TEMPORAL3 || c->tuning.kernel == FDTD_KERNEL_AUTO);
 }
 
+// Per-position coefficient arrays run the two-step kernel too, under AUTO or TEMPORAL (second order).
+bool use_full2(const fdtd_ctx *c) {
+    return c->coef_mode == COEF_FULL && c->order == 2 &&
+           (c->tuning.kernel == FDTD_KERNEL_AUTO || c->tuning.kernel == FDTD_KERNEL_TEMPORAL);
+}
+
 // Steps per launch of the context's multi-step kernel (use_temporal): 3 for TEMPORAL3, else 2.
 static int temporal_steps(const fdtd_ctx *c) { return c->tuning.kernel == FDTD_KERNEL_TEMPORAL3 ? 3 : 2; }
 
 // Tile kind of a context's one-step launches: 0 (Eq. 2) or 2 (fourth order).
 int one_step_kind(const fdtd_ctx *c) { return c->order == 4 ? 2 : 0; }
 
-// One launch of a single context (no graph): kinds 0 and 2 advance one step, kind 1 two steps.
+// One launch of a single context (no graph): kinds 0 and 2 advance one step, kinds 1 and 4 two steps, kind 3
+// three.
 int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
-    if (!use_fused(c)) {
+    if (!use_fused(c) && kind != 4) {
         if (c->order == 4)
             CK(c, launch_simple4_step(c->storage, make_desc(c, 0), c->cur, c->stream));
         else
             CK(c, launch_simple_step(c->storage, make_desc(c, 0), c->cur, c->stream));
         return FDTD_OK;
     }
-    Shape s = resolve_shape(c->storage, c->tuning, kind);
+    Shape s = resolve_shape(c->storage, c->tuning, kind, !c->ch_uniform);
     const fdtd_ctx::TileList &tl = c->tl[kind];
     FusedLaunch L{};
     L.recs = tl.d;
@@ -198,7 +215,7 @@ int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
     L.coef_class = coef_class_of(c->coef_mode, c->ch_uniform, kind == 1 && c->id_pec);
     if (kind == 0)
         CK(c, launch_fused_step(c->storage, L, c->stream));
-    else if (kind == 1)
+    else if (kind == 1 || kind == 4)
         CK(c, launch_fused2_step(c->storage, L, c->stream));
     else if (kind == 3)
         CK(c, launch_fused3_step(c->storage, L, c->stream));
@@ -541,6 +558,22 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
             }
         } else {
             c->coef_mode = COEF_FULL;
+            // ch identical in every cell (per component): the two-step kernel then streams the ce arrays alone
+            c->ch_uniform = 1;
+            if (have_ch)
+                for (int a = 0; a < 3; ++a) {
+                    c->ch_s[a] = ch[a][0];
+                    for (int k = 0; k < nz && c->ch_uniform; ++k)
+                        for (int j = 0; j < ny && c->ch_uniform; ++j)
+                            for (int i = 0; i < nx; ++i)
+                                if (ch[a][cidx(i, j, k)] != c->ch_s[a]) {
+                                    c->ch_uniform = 0;
+                                    break;
+                                }
+                }
+            if ((e = dmalloc(c, (void **)&c->coef_full[0], 6 * c->arr_elems * 4)) != cudaSuccess)
+                return cfail("coef alloc", e);
+            for (int a = 1; a < 6; ++a) c->coef_full[a] = c->coef_full[0] + a * c->arr_elems;
             std::vector<float> row((size_t)c->pitch * ny * nz, 0.f);
             for (int a = 0; a < 6; ++a) {
                 for (int k = 0; k < nz; ++k)
@@ -550,8 +583,6 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
                             const float v = a < 3 ? (have_ce ? ce[a][q] : vac) : (have_ch ? ch[a - 3][q] : vac);
                             row[((size_t)k * ny + j) * c->pitch + i] = v;
                         }
-                if ((e = dmalloc(c, (void **)&c->coef_full[a], row.size() * 4)) != cudaSuccess)
-                    return cfail("coef alloc", e);
                 if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cfail("sync", e);
                 if ((e = cudaMemcpy(c->coef_full[a], row.data(), row.size() * 4, cudaMemcpyHostToDevice)) !=
                     cudaSuccess)
@@ -590,12 +621,12 @@ void fdtd_destroy(fdtd_ctx *c) {
         pool_free(c->face[q], st);
         pool_free(c->face_ch[q], st);
     }
-    for (int a = 0; a < 6; ++a) pool_free(c->coef_full[a], st);
+    pool_free(c->coef_full[0], st);   // the six arrays share one allocation
     for (void *p : {(void *)c->id, (void *)c->id_pec, (void *)c->table_pec, (void *)c->table, (void *)c->inv_table,
                     (void *)c->table_fused,
                     (void *)c->d_status, (void *)c->d_partial, (void *)c->d_out, (void *)c->d_stage,
                     (void *)c->d_max, (void *)c->d_maps, (void *)c->d_desc, (void *)c->tl[0].d,
-                    (void *)c->tl[1].d, (void *)c->tl[2].d, (void *)c->tl[3].d, (void *)c->d_src_comp, (void *)c->d_src_off, (void *)c->d_wave,
+                    (void *)c->tl[1].d, (void *)c->tl[2].d, (void *)c->tl[3].d, (void *)c->tl[4].d, (void *)c->d_src_comp, (void *)c->d_src_off, (void *)c->d_wave,
                     (void *)c->d_probe_comp, (void *)c->d_probe_off, (void *)c->d_probe_buf, (void *)c->d_xclock})
         pool_free(p, st);
     pool_free(c->d_stage2, st);
@@ -643,7 +674,7 @@ int fdtd_set_tuning(fdtd_ctx *c, const fdtd_tuning *t) {
     if (n.stages == 3 && c->order == 4) return fail(c, FDTD_ERR_ARG, "the fourth-order kernel needs stages >= 4");
     if (n.zchunk < 0 || n.ctas_per_sm < 0) return fail(c, FDTD_ERR_ARG, "negative tuning value");
     c->tuning = n;
-    c->tl[0].key = c->tl[1].key = c->tl[2].key = c->tl[3].key = 0;   // force tile rebuilds
+    for (auto &tl : c->tl) tl.key = 0;   // force tile rebuilds
     cudaStreamSynchronize(c->stream);   // no graph of this context may still be running
     drop_graphs(c->graphs);
     return FDTD_OK;
@@ -729,7 +760,7 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
                 CK(c, cudaStreamSynchronize(c->stream));
             }
         }
-        c->tl[0].key = c->tl[1].key = c->tl[2].key = c->tl[3].key = 0;   // tile records embed the folded coefficients
+        for (auto &tl : c->tl) tl.key = 0;   // tile records embed the folded coefficients
         cudaStreamSynchronize(c->stream);
         drop_graphs(c->graphs);
     }
@@ -919,8 +950,9 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
     if (int rc = slab_check_steps(c, nsteps)) return rc;
     const bool fused = use_fused(c);
     const bool extras = extras_on(c);
+    const bool full2 = use_full2(c) && !extras;
     // currents enter between the E update of one step and the H update of the next: one step per launch
-    const bool temporal = use_temporal(c) && !extras;
+    const bool temporal = (use_temporal(c) && !extras) || full2;
     const int k1 = one_step_kind(c);
     int left = nsteps;
     if (c->inject_us <= 0)
@@ -935,8 +967,8 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
     if (left == 0) return FDTD_OK;
     if (fused)
         if (int rc = build_tiles(c, k1)) return rc;
-    // kind 1 (two steps per launch) or 3 (three steps per launch)
-    const int tkind = temporal_steps(c) == 3 ? 3 : 1, tper = temporal_steps(c);
+    // kind 1 (two steps per launch), 3 (three steps per launch) or 4 (two steps, per-position coefficients)
+    const int tkind = full2 ? 4 : temporal_steps(c) == 3 ? 3 : 1, tper = full2 ? 2 : temporal_steps(c);
     if (temporal)
         if (int rc = build_tiles(c, tkind)) return rc;
     // one launch from copy `parity` (fused kernels write copy parity ^ 1; the unfused one works in
@@ -958,8 +990,8 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
     const int kind = temporal ? tkind : k1;
     const int per = temporal ? tper : 1;
     const int K = per == 3 ? 18 : 16;   // steps per graph: an even number of launches
-    if (c->tuning.use_graph && fused && c->stream != nullptr && left >= K) {
-        GraphKey key{K, c->cur, kind + (extras ? 4 : 0)};
+    if (c->tuning.use_graph && (fused || full2) && c->stream != nullptr && left >= K) {
+        GraphKey key{K, c->cur, kind + (extras ? 8 : 0)};
         auto it = c->graphs.find(key);
         if (it == c->graphs.end()) {
             cudaGraph_t g;

@@ -29,7 +29,8 @@ constexpr int kMaxTable = 256;
 constexpr int kMaxPecMaterials = (kMaxTable - 1) / 8;   // 31: 1 + 8 x materials table entries
 constexpr int kTileX = 64;         // fused kernel tile width along x (cells)
 constexpr int kMapsPerCavity = 13; // [parity 0: 6 fields][parity 1: 6 fields][id]
-constexpr int kMapSets = 4;        // box sets: one-step, two-step, fourth-order and three-step kernels
+constexpr int kMapSets = 5;        // box sets: one-step, two-step, fourth-order, three-step kernels, and the two-step
+                                   // kernel with per-position coefficients (whose map 12 covers those arrays)
 
 template <typename T> struct Storage;
 template <> struct Storage<float> {

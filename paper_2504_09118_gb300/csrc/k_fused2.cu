@@ -30,7 +30,11 @@
 // faces a cell lies on select a table entry whose tangential E coefficients are zero, and entry 0,
 // read outside the cavity, has ce = 0) the steady planes apply no masks at all.  Every value keeps
 // the operation sequence of the one-step kernel: a masked coefficient there is the same zero in the
-// same fused multiply-add.  The kernel is compiled per coefficient class (CoefClass), so a single
+// same fused multiply-add.  Per-position coefficients (COEF_CLASS_FULL*) arrive as FP32 boxes in the unit,
+// 12 (ce) or 24 (ce and ch) bytes per cell and launch, with 12-row tiles so that a lane has the registers to
+// carry them a plane; HBM-side bound like the others.  160 x 150 x 140 FP32, ce varying: 24.7 us a step
+// (60 B per cell and two steps: 4.1 TB/s, from L2 in part) against 77 us for the unfused kernels (96 B a
+// step and latency-bound).  The kernel is compiled per coefficient class (CoefClass), so a single
 // cavity's launch tests its coefficient layout nowhere; batches keep a runtime class and the general
 // body.
 #include <type_traits>
@@ -81,17 +85,24 @@ template <typename T, int TY> __host__ __device__ constexpr int box_bytes() {
 // box, a load of its own, starts at the next 128-byte boundary.
 template <typename T, int TY> __host__ __device__ constexpr int idbox_off() { return al(6 * box_bytes<T, TY>(), 128); }
 template <int TY> __host__ __device__ constexpr int idbox_bytes() { return Geom2<float>::IBX * (TY + 4); }
-template <typename T, int TY> __host__ __device__ constexpr int slot2_bytes() {
-    return al(idbox_off<T, TY>() + idbox_bytes<TY>(), 128);
+// Per-position coefficients (COEF_CLASS_FULL*): in place of the id box, the FP32 boxes of the ce (and ch) arrays,
+// from column x0 - 2 rounded down to 4.
+__host__ __device__ constexpr int coef_arrays(int cm) {
+    return cm == COEF_CLASS_FULL_UNIFORM_H ? 3 : cm == COEF_CLASS_FULL ? 6 : 0;
+}
+constexpr int CBX = 68;
+template <int TY> __host__ __device__ constexpr int cbox_bytes() { return CBX * (TY + 4) * 4; }
+template <typename T, int TY, int CM = COEF_CLASS_ANY> __host__ __device__ constexpr int slot2_bytes() {
+    return al(idbox_off<T, TY>() + (coef_arrays(CM) ? coef_arrays(CM) * cbox_bytes<TY>() : idbox_bytes<TY>()), 128);
 }
 constexpr int PW = 68;   // shared plane row pitch: column x - x0 + 4 (lane cells at 2 lane + 2, + 3)
 template <int TY> __host__ __device__ constexpr int PR() { return TY + 5; }   // rows: r + 1 for r in -1 .. TY+3
 template <int TY> __host__ __device__ constexpr int plane_floats() { return PR<TY>() * PW; }
 constexpr int TAB2_BYTES = kMaxTable * 2 * 16;
-template <typename T, int TY> __host__ __device__ constexpr int smem2_bytes(int stages) {
+template <typename T, int TY, int CM = COEF_CLASS_ANY> __host__ __device__ constexpr int smem2_bytes(int stages) {
     // barriers/abort | records | table | H1 (Hx,Hz) | H2 (Hx,Hz) | E1 (Ex,Ez) x 2 | ring
     return 256 + NTR2 * (int)sizeof(TileRec) + TAB2_BYTES + al(8 * plane_floats<TY>() * 4, 128) +
-           stages * slot2_bytes<T, TY>();
+           stages * slot2_bytes<T, TY, CM>();
 }
 template <int TY> __host__ __device__ constexpr int threads2() { return (TY + 4) * 32; }
 
@@ -114,6 +125,11 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
     // PEC-coded ids (COEF_CLASS_PEC_*): the table zeroes the E coefficients on the faces and outside the
     // cavity (where the box read E = 0, so fma(0, curl, 0) = +0), so the steady planes need no masks
     constexpr bool PEC_TABLE = CM == COEF_CLASS_PEC_ID_UNIFORM_H || CM == COEF_CLASS_PEC_ID;
+    // per-position coefficients: the boxes hold 0 outside the cavity (TMA fill), so E stays 0 there; the walls'
+    // tangential components are masked.  A unit is released before E2 and H2 of its plane, so a lane carries
+    // its coefficients to the next plane (12-row tiles leave 128 registers a thread).
+    constexpr int NCO = coef_arrays(CM);
+    constexpr bool FULLC = NCO > 0, FULL_H = CM == COEF_CLASS_FULL;
 
     extern __shared__ __align__(128) unsigned char smem[];
     if (smem_u32(smem) & 127u) {
@@ -183,17 +199,19 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const int kk = kb + k;
                 if (lane == 0) {
                     const int src_copy = P.parity ^ rec->parity_off;
-                    const bool has_id = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H;
+                    const bool has_id = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
                     unsigned char *dst = slots + s * SB;
                     fence_proxy_async_smem();
                     if (tma_x_ok(P.status, G::box_x(rec->x0), (int)sizeof(T)) &&
                         (!has_id || tma_x_ok(P.status, rec->id_x0, 1))) {
-                        mbar_arrive_expect_tx(&full[s], 6 * FB + (has_id ? idbox_bytes<TY>() : 0));
+                        mbar_arrive_expect_tx(&full[s], 6 * FB + (has_id ? idbox_bytes<TY>() : 0) + NCO * cbox_bytes<TY>());
                         // the six field boxes in one load: a 4-D box (x, y, plane, field) lands as six
                         // consecutive FB-byte boxes
                         tma_load_4d(dst, rec->maps + src_copy * 6, G::box_x(rec->x0), rec->y0 - 2, kk, 0, &full[s]);
                         if (has_id)
                             tma_load_3d(dst + IDO, rec->maps + 12, rec->id_x0, rec->y0 - 2, kk, &full[s]);
+                        if (FULLC)
+                            tma_load_4d(dst + IDO, rec->maps + 12, (rec->x0 - 2) & ~3, rec->y0 - 2, kk, 0, &full[s]);
                     } else {
                         mbar_arrive(&full[s]);   // checked build: the unit is skipped, the slot still completes
                     }
@@ -240,7 +258,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
         const int bx = (x0 - 2) - G::box_x(x0) + 2 * lane;   // box column of the lane's first cell
         const int nx = rec->nx, ny = rec->ny, nz = rec->nz;
         const long long pitch = rec->pitch, plane = rec->plane;
-        const bool id_mode = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H;
+        const bool id_mode = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
         const bool ch_uni = CM == COEF_CLASS_ANY ? rec->ch_uniform != 0 : CM != COEF_CLASS_ID && CM != COEF_CLASS_PEC_ID;
         const int idoff = x0 - 2 - rec->id_x0;   // lane cells start this many bytes into the id box
         if (id_mode && rec->table != tab_cached) {
@@ -282,6 +300,20 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
         float2 e1px = zero2, e1py = zero2, e1pz = zero2;   // E1(j-1)
         float2 h2px = zero2, h2py = zero2;                 // H2(j-2) (Hx, Hy)
         uint32_t idprev = 0;                               // material ids of plane j-1
+        float2 cepx = zero2, cepy = zero2, cepz = zero2;   // FULLC: masked ce of plane j-1
+        float2 chpx = zero2, chpy = zero2, chpz = zero2;   // FULL_H: ch of plane j-1
+        // coefficient array a of plane k's unit on the lane's two cells, in storage units
+        const float coef_ratio = rec->ce[0], coef_iratio = rec->ce[1];   // s_E / s_H and its inverse (powers of two)
+        auto cload = [&](const unsigned char *slot, int a) {
+            float2 v = *reinterpret_cast<const float2 *>(slot + IDO + a * cbox_bytes<TY>() +
+                                                         4 * (by * CBX + 2 * lane + 2));
+            if (sizeof(T) == 2) {
+                const float f = a < 3 ? coef_ratio : coef_iratio;
+                v.x *= f;
+                v.y *= f;
+            }
+            return v;
+        };
 
         // One z-plane iteration.  ST (steady): k in [ks, kz1), where every phase runs, no mask depends on
         // k, and a failed ring wait only drops the stores: the phases then read a stale slot (in bounds)
@@ -308,7 +340,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
             float *e1cur = e1b + (k & 1) * 2 * PF, *e1prv = e1b + ((k + 1) & 1) * 2 * PF;
 
             // ---------------- phase 1: H1(k) on the lane's two cells
-            float2 e0x, e0y, e0z, h1x_, h1y_, h1z_;
+            float2 e0x, e0y, e0z, h1x_, h1y_, h1z_, chn_x = zero2, chn_y = zero2, chn_z = zero2;
             uint32_t idpair = 0;
             if (!ST) e0x = e0y = e0z = h1x_ = h1y_ = h1z_ = zero2;
             if (run) {
@@ -327,7 +359,16 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 // idoff is even (x0 and the 16-byte id box origin are), so the lane's two ids are one aligned u16
                 if (id_mode) idpair = *reinterpret_cast<const uint16_t *>(ida + by * G::IBX + idoff + 2 * lane);
                 float4 ca, cb;
-                coef(idpair, 1, ca, cb);
+                if (FULL_H) {
+                    const float2 cx = cload(slots + sa * SB, 3), cy = cload(slots + sa * SB, 4), cz = cload(slots + sa * SB, 5);
+                    ca = make_float4(cx.x, cy.x, cz.x, 0.f);
+                    cb = make_float4(cx.y, cy.y, cz.y, 0.f);
+                    chn_x = cx;
+                    chn_y = cy;
+                    chn_z = cz;
+                } else {
+                    coef(idpair, 1, ca, cb);
+                }
                 const float2 ez_x1 = make_float2(e0z.y, ez_x2), ey_x1 = make_float2(e0y.y, ey_x2);
                 h1x_ = fma2(make_float2(ca.x, cb.x), sub2(sub2(eyb, e0y), sub2(ez_y1, e0z)), h1x_);
                 h1y_ = fma2(make_float2(ca.y, cb.y), sub2(sub2(ez_x1, e0z), sub2(exb, e0x)), h1y_);
@@ -339,7 +380,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
 
             // ---------------- phase 2: E1(k) (zero outside the cavity: tangential at its far faces)
             // (in ST, a row that skips a phase leaves its pairs unset: no later phase of that row reads them)
-            float2 e1x, e1y, e1z;
+            float2 e1x, e1y, e1z, cen_x = zero2, cen_y = zero2, cen_z = zero2;
             if (!ST) e1x = e1y = e1z = zero2;
             if (run && do_e1 && r >= 1) {
                 const float2 hx_ym = *reinterpret_cast<const float2 *>(sh1x + (pr - 1) * PW + pc);
@@ -347,7 +388,13 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const float hz_xm = __shfl_up_sync(0xffffffffu, h1z_.y, 1);
                 const float hy_xm = __shfl_up_sync(0xffffffffu, h1y_.y, 1);
                 float4 ca, cb;
-                coef(idpair, 0, ca, cb);
+                if (FULLC) {
+                    const float2 cx = cload(slots + sa * SB, 0), cy = cload(slots + sa * SB, 1), cz = cload(slots + sa * SB, 2);
+                    ca = make_float4(cx.x, cy.x, cz.x, 0.f);
+                    cb = make_float4(cx.y, cy.y, cz.y, 0.f);
+                } else {
+                    coef(idpair, 0, ca, cb);
+                }
                 const bool inz = ST || k < nz, k1 = ST || k >= 1, j1 = gj >= 1;
                 const bool va = rowin && ina && inz, vb = rowin && inb && inz;
                 const bool i1a = gi >= 1;
@@ -361,8 +408,11 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 e1x = fma2(cex, sub2(sub2(h1z_, hz_ym), sub2(h1y_, h1py)), e0x);
                 e1y = fma2(cey, sub2(sub2(h1x_, h1px), sub2(h1z_, make_float2(hz_xm, h1z_.x))), e0y);
                 e1z = fma2(cez, sub2(sub2(h1y_, make_float2(hy_xm, h1y_.x)), sub2(h1x_, hx_ym)), e0z);
-                if (!NOMASK && !va) { e1x.x = 0.f; e1y.x = 0.f; e1z.x = 0.f; }
-                if (!NOMASK && !vb) { e1x.y = 0.f; e1y.y = 0.f; e1z.y = 0.f; }
+                cen_x = cex;
+                cen_y = cey;
+                cen_z = cez;
+                if (!NOMASK && !FULLC && !va) { e1x.x = 0.f; e1y.x = 0.f; e1z.x = 0.f; }
+                if (!NOMASK && !FULLC && !vb) { e1x.y = 0.f; e1y.y = 0.f; e1z.y = 0.f; }
                 *reinterpret_cast<float2 *>(e1cur + pr * PW + pc) = e1x;
                 *reinterpret_cast<float2 *>(e1cur + PF + pr * PW + pc) = e1z;
                 // one step: (H1, E1) is the result
@@ -392,7 +442,12 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const float ey_x2 = __shfl_down_sync(0xffffffffu, e1py.x, 1);
                 const float ez_x2 = __shfl_down_sync(0xffffffffu, e1pz.x, 1);
                 float4 ca, cb;
-                coef(idprev, 1, ca, cb);
+                if (FULL_H) {
+                    ca = make_float4(chpx.x, chpy.x, chpz.x, 0.f);
+                    cb = make_float4(chpx.y, chpy.y, chpz.y, 0.f);
+                } else {
+                    coef(idprev, 1, ca, cb);
+                }
                 const float2 ez_x1 = make_float2(e1pz.y, ez_x2), ey_x1 = make_float2(e1py.y, ey_x2);
                 h2x = fma2(make_float2(ca.x, cb.x), sub2(sub2(e1y, e1py), sub2(ez_y1, e1pz)), h1px);
                 h2y = fma2(make_float2(ca.y, cb.y), sub2(sub2(ez_x1, e1pz), sub2(e1x, e1px)), h1py);
@@ -410,15 +465,15 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const float2 hx_ym = *reinterpret_cast<const float2 *>(sh2x + (pr - 1) * PW + pc);
                 const float2 hz_ym = *reinterpret_cast<const float2 *>(sh2z + (pr - 1) * PW + pc);
                 float4 ca, cb;
-                coef(idprev, 0, ca, cb);
+                if (!FULLC) coef(idprev, 0, ca, cb);
                 const int kk = k - 1;
                 const bool k1 = ST || kk >= 1, j1 = gj >= 1, i1a = gi >= 1;
                 constexpr bool NOMASK = ST && PEC_TABLE;
-                const float2 cex = NOMASK ? make_float2(ca.x, cb.x)
+                const float2 cex = FULLC ? cepx : NOMASK ? make_float2(ca.x, cb.x)
                                           : make_float2((j1 && k1) ? ca.x : 0.f, (j1 && k1) ? cb.x : 0.f);
-                const float2 cey = NOMASK ? make_float2(ca.y, cb.y)
+                const float2 cey = FULLC ? cepy : NOMASK ? make_float2(ca.y, cb.y)
                                           : make_float2((i1a && k1) ? ca.y : 0.f, k1 ? cb.y : 0.f);
-                const float2 cez = NOMASK ? make_float2(ca.z, cb.z)
+                const float2 cez = FULLC ? cepz : NOMASK ? make_float2(ca.z, cb.z)
                                           : make_float2((i1a && j1) ? ca.z : 0.f, j1 ? cb.z : 0.f);
                 const float2 e2x = fma2(cex, sub2(sub2(h2z, hz_ym), sub2(h2y, h2py)), e1px);
                 const float2 e2y = fma2(cey, sub2(sub2(h2x, h2px), sub2(h2z, make_float2(h2z_xm, h2z.x))), e1py);
@@ -443,6 +498,16 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
             e1py = e1y;
             e1pz = e1z;
             idprev = idpair;
+            if (FULLC) {
+                cepx = cen_x;
+                cepy = cen_y;
+                cepz = cen_z;
+            }
+            if (FULL_H) {
+                chpx = chn_x;
+                chpy = chn_y;
+                chpz = chn_z;
+            }
             // ---------------- release unit k (and k+1 after the last plane)
             const bool last = !ST && k == kz1;
             __syncwarp();
@@ -477,7 +542,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
 
 template <typename T, int TY, bool BATCH, int CM>
 cudaError_t launch2_typed(const FusedLaunch &L, cudaStream_t s) {
-    const int smem = smem2_bytes<T, TY>(L.stages);
+    const int smem = smem2_bytes<T, TY, CM>(L.stages);
     auto kern = fused2_step_kernel<T, TY, BATCH, CM>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -489,7 +554,7 @@ cudaError_t launch2_typed(const FusedLaunch &L, cudaStream_t s) {
     P.parity = L.parity;
     P.status = L.status;
     P.stages = L.stages;
-    P.slot_bytes = slot2_bytes<T, TY>();
+    P.slot_bytes = slot2_bytes<T, TY, CM>();
     P.first = L.first;
     kern<<<L.grid, threads2<TY>(), smem, s>>>(P);
     return cudaGetLastError();
@@ -531,6 +596,21 @@ int fused2_smem_bytes(int storage, int tile_y, int stages) {
     return r;
 }
 
+int fused2_full_smem_bytes(int storage, int coef_class, int stages) {
+    if (coef_class == COEF_CLASS_FULL)
+        return storage == 0 ? smem2_bytes<float, kFullTileY, COEF_CLASS_FULL>(stages)
+                            : smem2_bytes<__half, kFullTileY, COEF_CLASS_FULL>(stages);
+    return storage == 0 ? smem2_bytes<float, kFullTileY, COEF_CLASS_FULL_UNIFORM_H>(stages)
+                        : smem2_bytes<__half, kFullTileY, COEF_CLASS_FULL_UNIFORM_H>(stages);
+}
+
+template <int CM> static cudaError_t launch2_full(int storage, const FusedLaunch &L, cudaStream_t s) {
+    if (L.tile_y != kFullTileY) return cudaErrorInvalidValue;
+    if (storage == 0) return launch2_typed<float, kFullTileY, false, CM>(L, s);
+    if (storage == 1) return launch2_typed<__half, kFullTileY, false, CM>(L, s);
+    return launch2_typed<__nv_bfloat16, kFullTileY, false, CM>(L, s);
+}
+
 cudaError_t fused2_occupancy(int storage, int tile_y, int stages, int *ctas_per_sm) {
     cudaError_t e = cudaErrorInvalidValue;
     FDTD_DISPATCH2(storage, tile_y, e = occupancy2_typed<T, TY>(stages, ctas_per_sm));
@@ -542,6 +622,8 @@ cudaError_t launch_fused2_step(int storage, const FusedLaunch &L, cudaStream_t s
     if (L.ntiles <= 0) return cudaSuccess;
     if (L.stages < 3 || L.stages > 8) return cudaErrorInvalidValue;
     cudaError_t e = cudaErrorInvalidValue;
+    if (L.coef_class == COEF_CLASS_FULL) return launch2_full<COEF_CLASS_FULL>(storage, L, s);
+    if (L.coef_class == COEF_CLASS_FULL_UNIFORM_H) return launch2_full<COEF_CLASS_FULL_UNIFORM_H>(storage, L, s);
     if (L.step || L.launch_steps == 1)   // a batch launch (or a one-step store launch)
         FDTD_DISPATCH2(storage, L.tile_y, e = (launch2_typed<T, TY, true, COEF_CLASS_ANY>(L, s)));
     else if (L.coef_class == COEF_CLASS_SCALAR)

@@ -54,6 +54,9 @@ enum CoefClass : int {
     // COEF_ID8 whose ids and table code the PEC faces (fdtd_ctx::id_pec): no per-cell masks in the kernel
     COEF_CLASS_PEC_ID_UNIFORM_H = 4,
     COEF_CLASS_PEC_ID = 5,
+    // COEF_FULL: per-position FP32 ce arrays (and ch arrays) streamed with the fields
+    COEF_CLASS_FULL_UNIFORM_H = 6,
+    COEF_CLASS_FULL = 7,
 };
 inline int coef_class_of(int coef_mode, int ch_uniform, bool pec_ids) {
     if (coef_mode == COEF_SCALAR) return COEF_CLASS_SCALAR;
@@ -61,6 +64,7 @@ inline int coef_class_of(int coef_mode, int ch_uniform, bool pec_ids) {
         if (pec_ids) return ch_uniform ? COEF_CLASS_PEC_ID_UNIFORM_H : COEF_CLASS_PEC_ID;
         return ch_uniform ? COEF_CLASS_ID_UNIFORM_H : COEF_CLASS_ID;
     }
+    if (coef_mode == COEF_FULL) return ch_uniform ? COEF_CLASS_FULL_UNIFORM_H : COEF_CLASS_FULL;
     return COEF_CLASS_ANY;
 }
 // Shared memory bytes and max co-resident CTAs per SM for a fused configuration.
@@ -117,6 +121,9 @@ cudaError_t launch_step_counter(long long *counter, int inc, cudaStream_t s);
 // Two-step (temporal blocking) kernel: output tile width along x, shared memory, occupancy, launch.
 int fused2_tile_w(int storage);
 int fused2_smem_bytes(int storage, int tile_y, int stages);
+// The same for per-position coefficients (tile height 12 only; the class is one of COEF_CLASS_FULL*).
+constexpr int kFullTileY = 12;
+int fused2_full_smem_bytes(int storage, int coef_class, int stages);
 cudaError_t fused2_occupancy(int storage, int tile_y, int stages, int *ctas_per_sm);
 cudaError_t launch_fused2_step(int storage, const FusedLaunch &L, cudaStream_t s);
 // The two-step kernel with two rows per consumer warp (k_fused2r.cu; tile heights 12 and 16): the same

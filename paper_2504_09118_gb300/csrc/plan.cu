@@ -6,12 +6,20 @@
 namespace fdtd {
 
 // Launch shape of kernel kind 0 (one step) or 1 (two steps) from the tuning (invalid fields -> defaults).
-Shape resolve_shape(int storage, const fdtd_tuning &t, int kind) {
+Shape resolve_shape(int storage, const fdtd_tuning &t, int kind, bool full_ch) {
     static std::mutex mu;
     static std::map<int, int> occ_cache;   // (kind, storage, tile_y, stages) -> max CTAs per SM
     Shape s;
     s.kind = kind;
     s.rows_per_warp = kind == 1 ? two_step_rows(t) : 1;
+    if (kind == 4) {   // one tile height; the deepest ring that fits (at least 3 slots), one CTA per SM
+        s.tile_y = kFullTileY;
+        const int cls = full_ch ? COEF_CLASS_FULL : COEF_CLASS_FULL_UNIFORM_H;
+        s.stages = (t.stages >= 3 && t.stages <= 8) ? t.stages : 6;
+        while (s.stages > 3 && fused2_full_smem_bytes(storage, cls, s.stages) > 227 * 1024) --s.stages;
+        s.ctas_per_sm = 1;
+        return s;
+    }
     const bool rows2 = s.rows_per_warp == 2;
     if (kind == 2)
         s.tile_y = (t.tile_y == 4 || t.tile_y == 8 || t.tile_y == 12 || t.tile_y == 16) ? t.tile_y : 12;
@@ -163,6 +171,10 @@ TileRec base_rec(const fdtd_ctx *c, int parity_off, int set) {
     const bool pec = set == 1 && c->id_pec;
     r.table = reinterpret_cast<const float4 *>(pec ? c->table_pec : c->table_fused);
     r.ntab = pec ? c->ntab_pec : c->ntab;
+    if (set == 4) {   // per-position coefficients are stored unscaled: the kernel applies the ratios
+        r.ce[0] = re;
+        r.ce[1] = 1.0f / re;
+    }
     r.stop = LLONG_MAX;
     r.maps = c->d_maps + set * kMapsPerCavity;
     for (int f = 0; f < 6; ++f) {
@@ -177,7 +189,7 @@ TileRec base_rec(const fdtd_ctx *c, int parity_off, int set) {
 void append_tiles_plan(std::vector<TileRec> &v, const fdtd_ctx *c, int parity_off, int tile_y,
                        const std::vector<int> &plan, int kind) {
     const TileRec b = base_rec(c, parity_off, kind);
-    const int tw = kind == 1 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
+    const int tw = kind == 1 || kind == 4 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
     int z0 = 0;
     for (int len : plan) {
         for (int y0 = 0; y0 < c->ny; y0 += tile_y)
@@ -227,14 +239,14 @@ std::vector<TileRec> assign_tiles(const std::vector<TileRec> &v, int G, int prol
 }
 
 int build_tiles(fdtd_ctx *c, int kind) {
-    Shape s = resolve_shape(c->storage, c->tuning, kind);
+    Shape s = resolve_shape(c->storage, c->tuning, kind, !c->ch_uniform);
     fdtd_ctx::TileList &tl = c->tl[kind];
     if (tl.key == s.tile_y && tl.d && tl.grid) return FDTD_OK;
-    int rc = encode_maps(c, kind, s.tile_y + (kind == 0 ? 2 : kind == 1 ? 4 : 6));
+    int rc = encode_maps(c, kind, s.tile_y + (kind == 0 ? 2 : kind == 1 || kind == 4 ? 4 : 6));
     if (rc) return rc;
-    const int tw = kind == 1 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
+    const int tw = kind == 1 || kind == 4 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
     const long long cols = (long long)((c->nx + tw - 1) / tw) * ((c->ny + s.tile_y - 1) / s.tile_y);
-    const int prologue = kind == 0 ? 1 : kind == 1 ? 3 : kind == 3 ? 5 : 4;
+    const int prologue = kind == 0 ? 1 : kind == 1 || kind == 4 ? 3 : kind == 3 ? 5 : 4;
     const int G = (int)std::min<long long>((long long)num_sms() * s.ctas_per_sm, cols * c->nz);
     std::vector<TileRec> listed, v;
     std::vector<int> first;
