@@ -48,6 +48,14 @@ struct GraphKey {
 };
 
 
+// Launch shape of a fused kernel (plan.cu).
+struct Shape {
+    int kind;   // 0: one step per launch, 1: two steps per launch, 2: one fourth-order step, 3: three steps,
+                // 4: two steps per launch with per-position coefficients
+    int tile_y, stages, ctas_per_sm;
+    int rows_per_warp;   // kind 1: rows per consumer warp (1, or 2 for FDTD_KERNEL_TEMPORAL2)
+};
+
 }  // namespace fdtd
 
 // The C ABI's opaque handles are global-namespace types; their members use the library's types.
@@ -99,7 +107,9 @@ struct fdtd_ctx {
     struct TileList {
         TileRec *d = nullptr;   // records, followed by the per-CTA range offsets
         int *first = nullptr;   // inside the same allocation as d
-        int n = 0, grid = 0, key = 0;
+        int n = 0, grid = 0;
+        bool ready = false;     // false: the tuning or the folded coefficients changed since it was built
+        Shape shape;            // the launch shape it was built for
     } tl[5];                                // [0] one-step, [1] two-step, [2] fourth-order, [3] three-step kernel,
                                             // [4] two-step kernel with per-position coefficients
     // many steps per launch on chip (k_resident.cu; small cavities under AUTO): boxes per axis and, allocated
@@ -220,15 +230,10 @@ int ensure_stage(fdtd_ctx *c);
 int ensure_stage2(fdtd_ctx *c);
 
 // ---- launch planning (plan.cu)
-struct Shape {
-    int kind;   // 0: one step per launch, 1: two steps per launch, 2: one fourth-order step, 3: three steps,
-                // 4: two steps per launch with per-position coefficients
-    int tile_y, stages, ctas_per_sm;
-    int rows_per_warp;   // kind 1: rows per consumer warp (1, or 2 for FDTD_KERNEL_TEMPORAL2)
-};
 // Rows per consumer warp of the two-step kernel a tuning selects.
 inline int two_step_rows(const fdtd_tuning &t) { return t.kernel == FDTD_KERNEL_TEMPORAL2 ? 2 : 1; }
 Shape resolve_shape(int storage, const fdtd_tuning &t, int kind = 0, bool full_ch = false);
+Shape cavity_shape(const fdtd_ctx *c, int kind);
 int choose_zlen(long long cols, int nz, int grid, int zchunk, int prologue_planes);
 long long simulate_plan(const std::vector<int> &plan, long long cols, int G, int prologue);
 std::vector<int> plan_chunks(long long cols, int nz, int G, int prologue, int zchunk);

@@ -199,8 +199,8 @@ int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
             CK(c, launch_simple_step(c->storage, make_desc(c, 0), c->cur, c->stream));
         return FDTD_OK;
     }
-    Shape s = resolve_shape(c->storage, c->tuning, kind, !c->ch_uniform);
     const fdtd_ctx::TileList &tl = c->tl[kind];
+    const Shape &s = tl.shape;
     FusedLaunch L{};
     L.recs = tl.d;
     L.ntiles = tl.n;
@@ -674,7 +674,7 @@ int fdtd_set_tuning(fdtd_ctx *c, const fdtd_tuning *t) {
     if (n.stages == 3 && c->order == 4) return fail(c, FDTD_ERR_ARG, "the fourth-order kernel needs stages >= 4");
     if (n.zchunk < 0 || n.ctas_per_sm < 0) return fail(c, FDTD_ERR_ARG, "negative tuning value");
     c->tuning = n;
-    for (auto &tl : c->tl) tl.key = 0;   // force tile rebuilds
+    for (auto &tl : c->tl) tl.ready = false;   // force tile rebuilds
     cudaStreamSynchronize(c->stream);   // no graph of this context may still be running
     drop_graphs(c->graphs);
     return FDTD_OK;
@@ -760,7 +760,7 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
                 CK(c, cudaStreamSynchronize(c->stream));
             }
         }
-        for (auto &tl : c->tl) tl.key = 0;   // tile records embed the folded coefficients
+        for (auto &tl : c->tl) tl.ready = false;   // tile records embed the folded coefficients
         cudaStreamSynchronize(c->stream);
         drop_graphs(c->graphs);
     }

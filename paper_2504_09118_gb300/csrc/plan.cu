@@ -125,6 +125,9 @@ std::vector<int> plan_chunks(long long cols, int nz, int G, int prologue, int zc
     }
     long long best = -1;
     auto consider = [&](const std::vector<int> &p) {
+        // the CTAs' mean load bounds the makespan from below: most plans with more chunks need no simulation
+        const long long work = cols * (nz + (long long)p.size() * prologue);
+        if (best >= 0 && (work + G - 1) / G >= best) return;
         const long long t = simulate_plan(p, cols, G, prologue);
         if (best < 0 || t < best) {
             best = t;
@@ -238,10 +241,47 @@ std::vector<TileRec> assign_tiles(const std::vector<TileRec> &v, int G, int prol
     return out;
 }
 
+// Launch shape of a cavity's kernel of this kind.  The two-step kernel (one row per warp) picks the tile height
+// the tuning leaves open from the work split: the plan's makespan in plane-times, times the time a plane takes
+// with that height.  Measured per plane (us; 512^3, 256^3, 200 x 131 x 120): FP32 0.63, 0.62, 0.66 with 8 rows,
+// 0.89, 0.85, 0.87 with 12 and 1.23, 1.13, 1.17 with 16; 16-bit 0.57-0.60, 0.73-0.76, 0.92-0.95.  Taller tiles
+// recompute less halo but cut the cavity into fewer, larger pieces: per step, 16 against 12 rows, 200 x 131 x
+// 120 FP32 21.2 against 19.4 us, 384^3 262 against 246 us, 256^3 84.1 against 85.1 us, 512^3 608 against 593 us.
+// Ring depth left open, FP32: 16 rows 5 slots, 12 rows 6, the deepest that fit, but one less from kDeepRingCells
+// cells on, where the deeper ring makes the CTAs read more halo from DRAM (512^3: 4.07 against 3.61 GB a launch)
+// and run up to 40 % slower: 512^3 694 against 608 us (16 rows), 727 against 593 us (12); 448^3 447 against 411 and
+// 430 against 393 us; 512 x 512 x 256 (6.7e7 cells) still 288 against 301 and 284 against 293 us.
+Shape cavity_shape(const fdtd_ctx *c, int kind) {
+    constexpr long long kDeepRingCells = 75000000;
+    fdtd_tuning t = c->tuning;
+    if (kind == 1 && two_step_rows(t) == 1) {
+        const bool f32 = c->storage == FDTD_F32;
+        const long long cells = (long long)c->nx * c->ny * c->nz;
+        if (t.tile_y != 8 && t.tile_y != 12 && t.tile_y != 16) {
+            const double plane_us[3] = {f32 ? 0.62 : 0.58, f32 ? (cells < kDeepRingCells ? 0.86 : 0.89) : 0.75,
+                                        f32 ? (cells < kDeepRingCells ? 1.14 : 1.23) : 0.935};
+            const int tw = fused2_tile_w(c->storage);
+            double best = -1.0;
+            for (int q = 0; q < 3; ++q) {
+                const int ty = 8 + 4 * q;
+                const long long cols = (long long)((c->nx + tw - 1) / tw) * ((c->ny + ty - 1) / ty);
+                const int G = (int)std::min<long long>(num_sms(), cols * c->nz);
+                const double us = plane_us[q] * simulate_plan(plan_chunks(cols, c->nz, G, 3, t.zchunk), cols, G, 3);
+                if (best < 0 || us < best) {
+                    best = us;
+                    t.tile_y = ty;
+                }
+            }
+        }
+        if (t.stages == 0 && f32 && cells >= kDeepRingCells) t.stages = t.tile_y == 16 ? 4 : t.tile_y == 12 ? 5 : 6;
+    }
+    return resolve_shape(c->storage, t, kind, !c->ch_uniform);
+}
+
 int build_tiles(fdtd_ctx *c, int kind) {
-    Shape s = resolve_shape(c->storage, c->tuning, kind, !c->ch_uniform);
     fdtd_ctx::TileList &tl = c->tl[kind];
-    if (tl.key == s.tile_y && tl.d && tl.grid) return FDTD_OK;
+    if (tl.ready) return FDTD_OK;
+    const Shape s = cavity_shape(c, kind);
     int rc = encode_maps(c, kind, s.tile_y + (kind == 0 ? 2 : kind == 1 || kind == 4 ? 4 : 6));
     if (rc) return rc;
     const int tw = kind == 1 || kind == 4 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
@@ -276,7 +316,8 @@ int build_tiles(fdtd_ctx *c, int kind) {
     CK(c, cudaStreamSynchronize(c->stream));
     tl.n = (int)v.size();
     tl.grid = grid;
-    tl.key = s.tile_y;
+    tl.shape = s;
+    tl.ready = true;
     return FDTD_OK;
 }
 
