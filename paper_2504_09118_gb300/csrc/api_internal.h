@@ -85,9 +85,11 @@ struct fdtd_ctx {
     int ntab_pec = 0;
     float *coef_full[6] = {};         // one allocation, arr_elems apart
     float scale[6] = {1, 1, 1, 1, 1, 1};
+    float folded_ratio = 1.f;         // the s_E / s_H that the device tables and tile records are folded for
     int cur = 0;
     long long steps = 0;
     bool has_fields = false;
+    bool launched = false;            // a kernel that can latch d_status has run on this context (never cleared)
     int *d_status = nullptr;
     double *d_partial = nullptr, *d_out = nullptr;
     float *d_stage = nullptr;    // canonical staging buffer for host transfers (lazy)
@@ -103,7 +105,6 @@ struct fdtd_ctx {
     CUtensorMap *d_maps = nullptr;          // kMapSets x kMapsPerCavity
     std::vector<CUtensorMap> host_maps[kMapSets];
     int maps_by[kMapSets] = {};   // box height each map set was encoded for (0: not yet)
-    CavityDesc *d_desc = nullptr;
     struct TileList {
         TileRec *d = nullptr;   // records, followed by the per-CTA range offsets
         int *first = nullptr;   // inside the same allocation as d
@@ -217,7 +218,6 @@ cudaError_t dmalloc(fdtd_ctx *c, void **p, size_t bytes);
 
 // ---- context helpers (ctx.cu)
 CavityDesc make_desc(const fdtd_ctx *c, int parity_off);
-int upload_desc(fdtd_ctx *c);
 int encode_maps(fdtd_ctx *c, int set, int box_y);
 void drop_graphs(std::map<GraphKey, cudaGraphExec_t> &g);
 bool use_fused(const fdtd_ctx *c);
@@ -225,7 +225,8 @@ bool use_temporal(const fdtd_ctx *c);
 bool use_full2(const fdtd_ctx *c);
 int one_step_kind(const fdtd_ctx *c);
 int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind = 0);
-int check_status(fdtd_ctx *c, int *d_status, cudaStream_t s);
+int check_status(fdtd_ctx *c, int *d_status, cudaStream_t s);   // waits for the stream
+int read_reductions(fdtd_ctx *c, const CavityDesc &d, int what, double out[3]);
 int ensure_stage(fdtd_ctx *c);
 int ensure_stage2(fdtd_ctx *c);
 

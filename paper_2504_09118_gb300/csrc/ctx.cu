@@ -85,12 +85,6 @@ CavityDesc make_desc(const fdtd_ctx *c, int parity_off) {
     return d;
 }
 
-int upload_desc(fdtd_ctx *c) {
-    CavityDesc d = make_desc(c, 0);
-    CK(c, cudaMemcpyAsync(c->d_desc, &d, sizeof d, cudaMemcpyHostToDevice, c->stream));
-    return FDTD_OK;
-}
-
 // Encode the 13 tensor maps of map set `set` (0: one-step kernel, 1: two-step kernel) for
 // boxes box_y rows high.  Set 1 sits right after set 0 in the context's map array.
 int encode_maps(fdtd_ctx *c, int set, int box_y) {
@@ -201,6 +195,7 @@ int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
     }
     const fdtd_ctx::TileList &tl = c->tl[kind];
     const Shape &s = tl.shape;
+    c->launched = true;
     FusedLaunch L{};
     L.recs = tl.d;
     L.ntiles = tl.n;
@@ -226,6 +221,10 @@ int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
 
 int check_status(fdtd_ctx *c, int *d_status, cudaStream_t s) {
     int h = 0;
+    if (d_status == c->d_status && !c->launched) {   // nothing can have latched it (a batch's launches latch the batch's)
+        CK(c, cudaStreamSynchronize(s));
+        return FDTD_OK;
+    }
     CK(c, cudaMemcpyAsync(&h, d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(c, cudaStreamSynchronize(s));
     if (h) {
@@ -236,6 +235,29 @@ int check_status(fdtd_ctx *c, int *d_status, cudaStream_t s) {
         return fail(c, FDTD_ERR_CUDA, "device status 0x%x", h);
     }
     return FDTD_OK;
+}
+
+// The three sums of launch_reductions on the host; the status word rides along, so one copy is waited for.
+int read_reductions(fdtd_ctx *c, const CavityDesc &d, int what, double out[3]) {
+    double o[4];
+    CK(c, launch_reductions(c->storage, d, c->cur, what, c->d_partial, reduction_blocks(), c->d_status, c->d_out, c->stream,
+                            c->order));
+    CK(c, cudaMemcpyAsync(o, c->d_out, sizeof o, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
+    for (int q = 0; q < 3; ++q) out[q] = o[q];
+    return o[3] == 0.0 ? FDTD_OK : check_status(c, c->d_status, c->stream);
+}
+
+// Small host arrays are read (and the smallest written) by the layout kernels themselves, where the GPU shares
+// the host's page tables (GB300: NVLink-C2C): six copies, their staging and events cost a small cavity more than
+// the bytes.  Above kDirectLoadBytes a load is limited by the link, and the copy engines' pipeline uses it better;
+// above kDirectStoreBytes an output may be fresh memory, whose pages a kernel's first touch maps much more slowly
+// than a copy does (1.6 MB: 5.6 against 1.9 ms).
+constexpr size_t kDirectLoadBytes = 16 << 20, kDirectStoreBytes = 1 << 20;
+static bool gpu_reads_host() {
+    int dev = 0, v = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) == cudaSuccess && v != 0;
 }
 
 int ensure_stage(fdtd_ctx *c) {
@@ -576,13 +598,13 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
             for (int a = 1; a < 6; ++a) c->coef_full[a] = c->coef_full[0] + a * c->arr_elems;
             std::vector<float> row((size_t)c->pitch * ny * nz, 0.f);
             for (int a = 0; a < 6; ++a) {
+                const float *src = a < 3 ? (have_ce ? ce[a] : nullptr) : (have_ch ? ch[a - 3] : nullptr);
                 for (int k = 0; k < nz; ++k)
-                    for (int j = 0; j < ny; ++j)
-                        for (int i = 0; i < nx; ++i) {
-                            const size_t q = cidx(i, j, k);
-                            const float v = a < 3 ? (have_ce ? ce[a][q] : vac) : (have_ch ? ch[a - 3][q] : vac);
-                            row[((size_t)k * ny + j) * c->pitch + i] = v;
-                        }
+                    for (int j = 0; j < ny; ++j) {
+                        float *dst = row.data() + ((size_t)k * ny + j) * c->pitch;
+                        if (src) memcpy(dst, src + cidx(0, j, k), (size_t)nx * sizeof(float));
+                        else std::fill(dst, dst + nx, vac);
+                    }
                 if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cfail("sync", e);
                 if ((e = cudaMemcpy(c->coef_full[a], row.data(), row.size() * 4, cudaMemcpyHostToDevice)) !=
                     cudaSuccess)
@@ -594,15 +616,10 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
     if ((e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream)) != cudaSuccess) return cfail("memset", e);
     const int nb = reduction_blocks();
     if ((e = dmalloc(c, (void **)&c->d_partial, sizeof(double) * 3 * nb)) != cudaSuccess) return cfail("alloc", e);
-    if ((e = dmalloc(c, (void **)&c->d_out, sizeof(double) * 3)) != cudaSuccess) return cfail("alloc", e);
+    if ((e = dmalloc(c, (void **)&c->d_out, sizeof(double) * 4)) != cudaSuccess) return cfail("alloc", e);
     if ((e = dmalloc(c, (void **)&c->d_max, sizeof(unsigned) * 6)) != cudaSuccess) return cfail("alloc", e);
     if ((e = dmalloc(c, (void **)&c->d_maps, sizeof(CUtensorMap) * kMapsPerCavity * kMapSets)) != cudaSuccess)
         return cfail("alloc", e);
-    if ((e = dmalloc(c, (void **)&c->d_desc, sizeof(CavityDesc))) != cudaSuccess) return cfail("alloc", e);
-    if (int rc = upload_desc(c)) {
-        g_create_error = c->err;
-        return bail(rc);
-    }
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cfail("sync", e);
     *out = c;
     return FDTD_OK;
@@ -625,7 +642,7 @@ void fdtd_destroy(fdtd_ctx *c) {
     for (void *p : {(void *)c->id, (void *)c->id_pec, (void *)c->table_pec, (void *)c->table, (void *)c->inv_table,
                     (void *)c->table_fused,
                     (void *)c->d_status, (void *)c->d_partial, (void *)c->d_out, (void *)c->d_stage,
-                    (void *)c->d_max, (void *)c->d_maps, (void *)c->d_desc, (void *)c->tl[0].d,
+                    (void *)c->d_max, (void *)c->d_maps, (void *)c->tl[0].d,
                     (void *)c->tl[1].d, (void *)c->tl[2].d, (void *)c->tl[3].d, (void *)c->tl[4].d, (void *)c->d_src_comp, (void *)c->d_src_off, (void *)c->d_wave,
                     (void *)c->d_probe_comp, (void *)c->d_probe_off, (void *)c->d_probe_buf, (void *)c->d_xclock})
         pool_free(p, st);
@@ -710,12 +727,16 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
         if (!f[q]) return fail(c, FDTD_ERR_ARG, "field %d is NULL", q);
     if (c->batch) return fail(c, FDTD_ERR_STATE, "context is a batch member; remove it first");
     const size_t n = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
-    if (!on_device)
+    // whether the kernels read f itself: device arrays, or small host arrays
+    const bool direct = on_device || (6 * n * 4 <= kDirectLoadBytes && gpu_reads_host());
+    if (!direct)
         if (int rc = ensure_stage(c)) return rc;
     // scales for 16-bit storage: s_c = 2^(8 - ceil(log2 max|F_c|))
     if (c->storage != FDTD_F32) {
+        const float old_scale[2] = {c->scale[0], c->scale[3]};
+        float new_scale[2];   // taken only when both groups pass their checks
         CK(c, cudaMemsetAsync(c->d_max, 0, sizeof(unsigned) * 6, c->stream));
-        if (on_device)
+        if (direct)
             CK(c, launch_maxabs(f, 0, 6, c->nx, c->ny, c->nz, c->d_max, c->stream));
         else
             for (int q = 0; q < 6; ++q) {
@@ -742,10 +763,13 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
                     return fail(c, FDTD_ERR_ARG, "fixed storage scale %g overflows FP16 for |%s| up to %g", sc,
                                 g ? "H" : "E", (double)mx);
             }
-            for (int q = 3 * g; q < 3 * g + 3; ++q) c->scale[q] = sc;
+            new_scale[g] = sc;
         }
-        if (c->table_fused) {
-            const float re = c->scale[0] / c->scale[3];
+        for (int q = 0; q < 6; ++q) c->scale[q] = new_scale[q / 3];
+        // the coefficients are folded with s_E / s_H only: nothing changes when this load's ratio is the last one's
+        const float re = c->scale[0] / c->scale[3];
+        const bool refold = re != c->folded_ratio;
+        if (refold && c->table_fused) {
             std::vector<float> tf = c->host_table;
             for (int n = 0; n < c->ntab; ++n)
                 for (int q = 0; q < 3; ++q) {
@@ -760,13 +784,17 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
                 CK(c, cudaStreamSynchronize(c->stream));
             }
         }
-        for (auto &tl : c->tl) tl.ready = false;   // tile records embed the folded coefficients
-        cudaStreamSynchronize(c->stream);
-        drop_graphs(c->graphs);
+        if (refold) {
+            for (auto &tl : c->tl) tl.ready = false;   // tile records embed the folded coefficients
+            c->folded_ratio = re;
+        }
+        if (refold || c->scale[0] != old_scale[0] || c->scale[3] != old_scale[1]) {
+            cudaStreamSynchronize(c->stream);   // graphs hold the tile records and, with currents or probes, the scales
+            drop_graphs(c->graphs);
+        }
     }
-    if (int rc = upload_desc(c)) return rc;
     CavityDesc d = make_desc(c, 0);
-    if (on_device) {
+    if (direct) {
         CK(c, launch_pack(c->storage, d, 0, 0, 6, f, c->stream));
     } else {
         // host fields: field q is copied into staging buffer q & 1 on the copy stream while the
@@ -790,12 +818,11 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
     if (c->d_probe_buf)
         CK(c, cudaMemsetAsync(c->d_probe_buf, 0, sizeof(float) * (size_t)c->nprobe * c->probe_cap, c->stream));
     c->probe_start = 0;
-    CK(c, cudaStreamSynchronize(c->stream));
     c->cur = 0;
     c->steps = 0;
     c->has_fields = true;
     slab_after_load(c);
-    return check_status(c, c->d_status, c->stream);
+    return check_status(c, c->d_status, c->stream);   // waits for the stream
 }
 
 int fdtd_prefetch_fields(fdtd_ctx *c, const float *const f[6]) {
@@ -844,18 +871,18 @@ int fdtd_get_fields(fdtd_ctx *c, float *const f[6], int on_device) {
         if (!f[q]) return fail(c, FDTD_ERR_ARG, "field %d is NULL", q);
     if (c->batch) return fail(c, FDTD_ERR_STATE, "context is a batch member; remove it first");
     const size_t n = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
-    if (!on_device)
+    const bool direct = on_device || (6 * n * 4 <= kDirectStoreBytes && gpu_reads_host());
+    if (!direct)
         if (int rc = ensure_stage(c)) return rc;
     CavityDesc d = make_desc(c, 0);
-    if (on_device)
+    if (direct)
         CK(c, launch_unpack(c->storage, d, c->cur, 0, 6, f, c->stream));
     else
         for (int q = 0; q < 6; ++q) {
             CK(c, launch_unpack(c->storage, d, c->cur, q, 1, &c->d_stage, c->stream));
             CK(c, cudaMemcpyAsync(f[q], c->d_stage, n * 4, cudaMemcpyDeviceToHost, c->stream));
         }
-    CK(c, cudaStreamSynchronize(c->stream));
-    return check_status(c, c->d_status, c->stream);
+    return check_status(c, c->d_status, c->stream);   // waits for the stream
 }
 
 // Steps a resident launch takes at least and at most.  A launch loads and stores the whole state, which a few
@@ -927,6 +954,7 @@ static int step_resident(fdtd_ctx *c, int n, bool *done) {
     P.epoch = reinterpret_cast<unsigned *>(static_cast<char *>(c->d_resident) + words);
     P.status = c->d_status;
     if (extras_on(c)) P.X = make_extras(c);
+    c->launched = true;
     const cudaError_t e = launch_resident(P, c->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
         cudaGetLastError();
@@ -1029,18 +1057,13 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
 
 int fdtd_sync(fdtd_ctx *c) {
     if (!c) return FDTD_ERR_ARG;
-    CK(c, cudaStreamSynchronize(c->stream));
     return check_status(c, c->d_status, c->stream);
 }
 
 static int run_reductions(fdtd_ctx *c, int what, double out[3]) {
     if (!c->has_fields) return fail(c, FDTD_ERR_STATE, "fdtd_set_fields has not been called");
     if (c->batch) return fail(c, FDTD_ERR_STATE, "context is a batch member; remove it first");
-    CK(c, launch_reductions(c->storage, make_desc(c, 0), c->cur, what, c->d_partial, reduction_blocks(), c->d_out,
-                            c->stream, c->order));
-    CK(c, cudaMemcpyAsync(out, c->d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
-    return check_status(c, c->d_status, c->stream);
+    return read_reductions(c, make_desc(c, 0), what, out);
 }
 
 int fdtd_energy(fdtd_ctx *c, double *W) {

@@ -415,14 +415,26 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const CavityDesc d,
     }
 }
 
-__global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double *partial, int nblocks, double *out) {
-    __shared__ double sh[kRedThreads / 32];
+// Sums of the block partials (in a fixed order) and the status word: one read-back for both.
+__global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double *partial, int nblocks, const int *status,
+                                                                   double *out) {
+    __shared__ double sh[3][kRedThreads / 32];
+    double v[3] = {0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nblocks; b += kRedThreads)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] += partial[3 * b + q];
+#pragma unroll
     for (int q = 0; q < 3; ++q) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += kRedThreads) v += partial[3 * b + q];
-        v = block_sum(v, sh);
-        if (threadIdx.x == 0) out[q] = v;
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = v[q];
     }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double r = 0.0;
+        for (int i = 0; i < kRedThreads / 32; ++i) r += sh[threadIdx.x][i];
+        out[threadIdx.x] = r;
+    }
+    if (threadIdx.x == 3) out[3] = (double)*status;
 }
 
 template <typename T>
@@ -487,7 +499,7 @@ cudaError_t launch_simple_step(int storage, const CavityDesc &d, int copy, cudaS
 int reduction_blocks() { return kRedBlocks; }
 
 cudaError_t launch_reductions(int storage, const CavityDesc &d, int copy, int what, double *partial, int nblocks,
-                              double *out, cudaStream_t s, int order) {
+                              const int *status, double *out, cudaStream_t s, int order) {
     if (order == 4) {
         cudaError_t e = launch_reductions4(storage, d, copy, what, partial, nblocks, s);
         if (e != cudaSuccess) return e;
@@ -495,7 +507,7 @@ cudaError_t launch_reductions(int storage, const CavityDesc &d, int copy, int wh
         FDTD_STORAGE_DISPATCH(storage, reduce_kernel<T, 0><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial));
     else
         FDTD_STORAGE_DISPATCH(storage, reduce_kernel<T, 1><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial));
-    reduce_final_kernel<<<1, kRedThreads, 0, s>>>(partial, nblocks, out);
+    reduce_final_kernel<<<1, kRedThreads, 0, s>>>(partial, nblocks, status, out);
     return cudaGetLastError();
 }
 

@@ -20,8 +20,9 @@ cudaError_t launch_simple_step(int storage, const CavityDesc &d, int copy, cudaS
 // Reductions accumulated in FP64: what == 0 gives out[0] = sum E^2/ce + H.(H - ch curl E)/ch;
 // what == 1 gives out[1] = sum divE^2, out[2] = sum divH^2.  partial holds nblocks*3 doubles.
 // order 4 takes the curl and divergences of the fourth-order scheme.
+// out[3] = the device status word.
 cudaError_t launch_reductions(int storage, const CavityDesc &d, int copy, int what, double *partial, int nblocks,
-                              double *out, cudaStream_t s, int order = 2);
+                              const int *status, double *out, cudaStream_t s, int order = 2);
 // Fourth-order scheme (k_order4.cu): one unfused step in place on copy `copy`, and the per-block
 // partials of its reductions (same layout as launch_reductions' partial).
 cudaError_t launch_simple4_step(int storage, const CavityDesc &d, int copy, cudaStream_t s);

@@ -196,11 +196,7 @@ static int slab_reduce(fdtd_ctx *c, int what, double out[3]) {
     d.kr_lo = c->slab.g_lo;
     d.kr_hi = c->nz - c->slab.g_hi;
     d.face_top = c->slab.g_hi == 0;
-    CK(c, launch_reductions(c->storage, d, c->cur, what, c->d_partial, reduction_blocks(), c->d_out, c->stream,
-                            c->order));
-    CK(c, cudaMemcpyAsync(out, c->d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
-    return check_status(c, c->d_status, c->stream);
+    return read_reductions(c, d, what, out);
 }
 
 int fdtd_slab_energy(fdtd_ctx *c, double *W) {

@@ -29,7 +29,11 @@ def _state(dims, seed=0):
     return full, kept
 
 
-@pytest.mark.parametrize("dims", SIZES)
+# host arrays just below and above the sizes up to which the kernels write (1 MiB) and read (16 MiB) them directly
+DIRECT = [(34, 34, 33), (35, 35, 35), (88, 88, 87), (88, 88, 88)]
+
+
+@pytest.mark.parametrize("dims", SIZES + DIRECT)
 @pytest.mark.parametrize("device", [False, True])
 def test_load_and_read_back_f32_exact(dims, device):
     import torch
@@ -82,3 +86,33 @@ def test_f16_scale_follows_the_largest_entry_of_the_extents(dims, where):
             ref = (ref * sc).astype(np.float16).astype(np.float32) / sc
             np.testing.assert_array_equal(dev[c], ref)
             np.testing.assert_array_equal(host[c], ref)
+
+
+@pytest.mark.parametrize("tuning", [{}, dict(kernel=2, use_graph=1), dict(kernel=3, use_graph=1)])
+@pytest.mark.parametrize("storage", [1, 2])
+def test_reloads_with_equal_and_other_scales_match_a_fresh_context(tuning, storage):
+    """The folded coefficients and launch records of a 16-bit context are rebuilt only when s_E / s_H changes: each of a
+    series of loads (another ratio, back, the same, both scales times 4 with a current set) steps as in a new context."""
+    import torch
+    from paper_2504_09118_gb300 import Cavity
+    dims = (61, 30, 21)
+    ce, ch = ci.sphere_coefficients(ci.sphere_list(9, 4, dims, 3.0, 9.0), *dims, ci.COURANT_HALF_DT)
+    base = ci.random_fields(31, *dims)
+    src = [(2, 30, 15, 10)], np.linspace(0.1, 1.0, 40, dtype=np.float32)[None]
+    s = torch.cuda.Stream()
+
+    def solve(cav, e, h, sources):
+        cav.set_sources(*(src if sources else ([], [])))
+        cav.set_fields([a * np.float32(e if c < 3 else h) for c, a in enumerate(base)])
+        cav.step(19)
+        return cav.get_fields()
+
+    with Cavity(*dims, ci.COURANT_HALF_DT, 1.0, ce, ch, storage, s) as cav:
+        cav.tune(**tuning)
+        for e, h, sources in ((1, 1, 0), (8, 1, 0), (1, 1, 0), (1, 1, 0), (1, 1, 1), (4, 4, 1), (1, 0.5, 1)):
+            got = solve(cav, e, h, sources)
+            with Cavity(*dims, ci.COURANT_HALF_DT, 1.0, ce, ch, storage, s) as fresh:
+                fresh.tune(**tuning)
+                want = solve(fresh, e, h, sources)
+            for a, b in zip(got, want):
+                np.testing.assert_array_equal(a, b)
