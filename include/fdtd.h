@@ -320,7 +320,8 @@ FDTD_API long long fdtd_batch_steps_done(const fdtd_batch *b);
  * result is bit-identical to stepping it alone with FP32 storage. */
 FDTD_API int fdtd_batch_step(fdtd_batch *b, int nsteps);
 
-/* fdtd_batch_set_tuning - launch shape for the batch kernel: FUSED (one step per launch) or TEMPORAL,
+/* fdtd_batch_set_tuning - launch shape for the batch kernel (tile_y 0: 12 rows for the two-step kernel, 16 for
+ * TEMPORAL2): FUSED (one step per launch) or TEMPORAL,
  * TEMPORAL2 or AUTO (two steps per launch; TEMPORAL3 is for single cavities: FDTD_ERR_ARG); may change
  * between fdtd_batch_step calls.  With one CTA per SM and every running member stopping at the same
  * clock, tiles are assigned to the CTAs on the host for balance; otherwise they are dealt round-robin. */

@@ -166,6 +166,8 @@ struct fdtd_batch {
     TileRec *d_tiles = nullptr;      // tile records, then (at d_first) the per-CTA range offsets
     int *d_first = nullptr;          // grid + 1 offsets when the tiles are assigned to CTAs on the host, else NULL
     int tiles_cap = 0, ntiles = 0, grid = 0;
+    Shape shape;                     // launch shape the tile list was built for
+    bool steady = false;             // two-step kernel: the instance with steady-state plane bodies
     // pinned staging of the tile-list uploads, two buffers used in turn: a copy from pageable memory may
     // wait for the stream, which would drain the queued launches at every change of membership
     void *h_stage[2] = {nullptr, nullptr};

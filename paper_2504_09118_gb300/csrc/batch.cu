@@ -161,13 +161,55 @@ static int batch_kind(const fdtd_batch *b) {
                : 0;
 }
 
+// Plane-times of the fullest CTA when the running members' tile columns are cut into pieces of at most zlen planes,
+// the pieces sorted longest first and given to the CTA that frees first (balanced) or dealt in turn.
+static long long batch_makespan(const std::vector<std::pair<int, long long>> &members, int zlen, int G, int prologue,
+                                bool balanced) {   // members: (nz, tile columns)
+    std::map<int, long long, std::greater<int>> pieces;   // length -> count
+    for (const auto &m : members) {
+        if (m.first >= zlen) pieces[zlen] += m.second * (m.first / zlen);
+        if (m.first % zlen) pieces[m.first % zlen] += m.second;
+    }
+    if (!balanced) {   // dealt in turn, CTA 0 gets the longest piece of every round
+        long long at = 0, next = 0, sum = 0;
+        for (const auto &p : pieces) {
+            at += p.second;
+            if (next < at) {
+                const long long rounds = (at - next + G - 1) / G;
+                sum += rounds * (p.first + prologue);
+                next += rounds * G;
+            }
+        }
+        return sum;
+    }
+    std::map<long long, long long> busy;   // finish time -> CTAs
+    busy[0] = G;
+    for (const auto &p : pieces) {
+        long long left = p.second;
+        while (left > 0) {
+            auto it = busy.begin();
+            const long long t = it->first, k = std::min(it->second, left);
+            if ((it->second -= k) == 0) busy.erase(it);
+            busy[t + p.first + prologue] += k;
+            left -= k;
+        }
+    }
+    return busy.rbegin()->first;
+}
+
 // Rebuild the packed tile list (asynchronously on the batch stream: the upload runs after the
 // launches already enqueued, and the old buffer is released in stream order).
 static int batch_rebuild(fdtd_batch *b) {
     if (!b->dirty) return FDTD_OK;
     batch_retire_graphs(b);
     const int kind = batch_kind(b);
-    Shape s = resolve_shape(b->storage, b->tuning, kind);
+    // The two-step kernel's default height for batches is 12 rows: the instance with steady-state plane bodies needs
+    // the 128 registers that leaves (with 16 rows it spills).  us per launch against 16 rows without them: 48 cavities
+    // of sides 16..96 FP32 184 -> 144, 24 with own step counts BF16 91 -> 75, 128 FP32 419 -> 347, 12 of sides 16..40
+    // 22.8 -> 21.7 (z-lengths by the rule below).
+    fdtd_tuning tuning = b->tuning;
+    if (kind == 1 && two_step_rows(tuning) == 1 && tuning.tile_y != 8 && tuning.tile_y != 16) tuning.tile_y = 12;
+    Shape s = resolve_shape(b->storage, tuning, kind);
     const int box_y = s.tile_y + (kind == 0 ? 2 : kind == 1 ? 4 : 6);
     const int G = num_sms() * s.ctas_per_sm;
     std::vector<TileRec> tiles;
@@ -181,6 +223,8 @@ static int batch_rebuild(fdtd_batch *b) {
     long long total_cols = 0;
     bool same_stop = true;   // every running member stops at the same clock (or never)
     long long stop0 = -1;
+    std::vector<std::pair<int, long long>> columns;   // (nz, tile columns) of each running member
+    int max_nz = 1;
     for (auto &mb : b->members) {
         if (mb.stop <= b->step) continue;   // finished members carry no tiles
         fdtd_ctx *c = mb.c;
@@ -188,17 +232,33 @@ static int batch_rebuild(fdtd_batch *b) {
         const long long cols = (long long)((c->nx + tw - 1) / tw) * ((c->ny + s.tile_y - 1) / s.tile_y);
         total_cols += cols;
         total_cols_planes += cols * c->nz;
+        columns.emplace_back(c->nz, cols);
+        max_nz = std::max(max_nz, c->nz);
         if (stop0 < 0) stop0 = mb.stop;
         same_stop = same_stop && mb.stop == stop0;
     }
     // tiles assigned to the CTAs on the host (below) when every tile takes part in every launch
     const bool balanced = s.ctas_per_sm == 1 && same_stop;
-    // One z-length for all members so tiles carry similar work: about 8 tiles per CTA; with balanced ranges
-    // and at least 4 tile columns per CTA, whole members (fewer tile prologues; 0.9 % faster on 256 members
-    // of sides 16..96)
-    const int zlen = b->tuning.zchunk > 0              ? b->tuning.zchunk
-                     : (balanced && total_cols >= 4LL * G) ? INT_MAX
-                                                         : (int)std::max<long long>(8, total_cols_planes / std::max(1, 8 * G));
+    // One z-length for all members.  Two-step kernel: the candidate with the shortest makespan, a tile costing its
+    // planes and four more (three that prime the recurrence, and their general plane body).  Measured against about 8
+    // tiles per CTA, 12 rows: 166 -> 144 us a launch (48 cavities FP32), 83 -> 75 us (24 BF16, own step counts).
+    // Not for 16 rows dealt in turn, where longer pieces measured better (128 BF16 cavities 378 against 360 us).
+    // Other kernels, and those: about 8 tiles per CTA; with balanced ranges and at least 4 tile columns per CTA, whole members.
+    int zlen = b->tuning.zchunk;
+    if (zlen <= 0 && kind == 1 && s.ctas_per_sm == 1 && (balanced || s.tile_y <= 12)) {
+        long long best = -1;
+        for (int z : {max_nz, 96, 64, 48, 32, 24, 16, 12, 8}) {
+            if (z > max_nz) continue;
+            const long long t = batch_makespan(columns, z, G, 4, balanced);
+            if (best < 0 || t < best) {
+                best = t;
+                zlen = z;
+            }
+        }
+    }
+    if (zlen <= 0)
+        zlen = (balanced && total_cols >= 4LL * G) ? INT_MAX
+                                                   : (int)std::max<long long>(8, total_cols_planes / std::max(1, 8 * G));
     for (auto &mb : b->members) {
         if (mb.stop <= b->step) continue;
         const size_t first = tiles.size();
@@ -256,6 +316,8 @@ static int batch_rebuild(fdtd_batch *b) {
     if (cudaEventRecord(b->h_stage_ev[si], b->stream) != cudaSuccess) return bfail(b, FDTD_ERR_CUDA, "event record");
     b->ntiles = (int)tiles.size();
     b->grid = grid;
+    b->shape = s;
+    b->steady = kind == 1 && s.rows_per_warp == 1 && s.tile_y <= 12;   // no instance with 16 rows
     b->dirty = false;
     return FDTD_OK;
 }
@@ -263,7 +325,7 @@ static int batch_rebuild(fdtd_batch *b) {
 // One launch advancing the batch clock by nsteps (1, or 2 with the two-step kernel), then the clock.
 static int batch_launch(fdtd_batch *b, int parity, int nsteps) {
     const int kind = batch_kind(b);
-    Shape s = resolve_shape(b->storage, b->tuning, kind);
+    const Shape &s = b->shape;
     FusedLaunch L{};
     L.recs = b->d_tiles;
     L.first = b->d_first;
@@ -276,6 +338,7 @@ static int batch_launch(fdtd_batch *b, int parity, int nsteps) {
     L.grid = b->grid;
     L.launch_steps = nsteps;
     L.rows_per_warp = s.rows_per_warp;
+    L.coef_class = b->steady ? COEF_CLASS_ANY_STEADY : COEF_CLASS_ANY;
     cudaError_t e = kind == 0   ? launch_fused_step(b->storage, L, b->stream)
                     : kind == 1 ? launch_fused2_step(b->storage, L, b->stream)
                                 : launch_fused4_step(b->storage, L, b->stream);

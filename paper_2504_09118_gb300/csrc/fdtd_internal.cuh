@@ -133,7 +133,8 @@ struct alignas(16) TileRec {
     int ntab;                    // COEF_ID8: table entries
     int nz;
     int id_x0;                   // two-step kernel: x origin of the id box (a multiple of 16)
-    int pad[13];
+    int pec;                     // two-step kernel: ids and table code the PEC faces
+    int pad[12];
 };
 static_assert(sizeof(TileRec) == 256, "TileRec must be 256 bytes");
 

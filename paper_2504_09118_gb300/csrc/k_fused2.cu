@@ -118,10 +118,12 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
     static_assert(FB % 16 == 0 && FE % 2 == 0, "field boxes keep 16-byte rows and even-aligned pairs");
     constexpr int NCW = TY + 3, NCT = NCW * 32;
     constexpr int PF = plane_floats<TY>();
-    // the steady-state plane body (below) for launches of one coefficient layout; a batch, whose
-    // instance also carries the stop-clock logic, runs every plane through the general body, which
-    // needs fewer registers (no spill at 16 rows)
-    constexpr bool SPLIT = !BATCH && CM != COEF_CLASS_ANY;
+    // the steady-state plane body (below) for launches of one coefficient layout; a batch of deep tiles, whose
+    // members may differ, holds two of them (PEC-coded ids, and a uniform cavity with masks) and picks one per
+    // tile (BSTEADY: 8 and 12 rows; with 16 the 96 registers make it spill)
+    constexpr bool ANYC = CM == COEF_CLASS_ANY || CM == COEF_CLASS_ANY_STEADY;
+    constexpr bool BSTEADY = BATCH && CM == COEF_CLASS_ANY_STEADY;
+    constexpr bool SPLIT = !BATCH && !ANYC;
     // PEC-coded ids (COEF_CLASS_PEC_*): the table zeroes the E coefficients on the faces and outside the
     // cavity (where the box read E = 0, so fma(0, curl, 0) = +0), so the steady planes need no masks
     constexpr bool PEC_TABLE = CM == COEF_CLASS_PEC_ID_UNIFORM_H || CM == COEF_CLASS_PEC_ID;
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const int kk = kb + k;
                 if (lane == 0) {
                     const int src_copy = P.parity ^ rec->parity_off;
-                    const bool has_id = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
+                    const bool has_id = ANYC ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
                     unsigned char *dst = slots + s * SB;
                     fence_proxy_async_smem();
                     if (tma_x_ok(P.status, G::box_x(rec->x0), (int)sizeof(T)) &&
@@ -258,8 +260,8 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
         const int bx = (x0 - 2) - G::box_x(x0) + 2 * lane;   // box column of the lane's first cell
         const int nx = rec->nx, ny = rec->ny, nz = rec->nz;
         const long long pitch = rec->pitch, plane = rec->plane;
-        const bool id_mode = CM == COEF_CLASS_ANY ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
-        const bool ch_uni = CM == COEF_CLASS_ANY ? rec->ch_uniform != 0 : CM != COEF_CLASS_ID && CM != COEF_CLASS_PEC_ID;
+        const bool id_mode = ANYC ? rec->mode == COEF_ID8 : CM >= COEF_CLASS_ID_UNIFORM_H && !FULLC;
+        const bool ch_uni = ANYC ? rec->ch_uniform != 0 : CM != COEF_CLASS_ID && CM != COEF_CLASS_PEC_ID;
         const int idoff = x0 - 2 - rec->id_x0;   // lane cells start this many bytes into the id box
         if (id_mode && rec->table != tab_cached) {
             const float4 *src = rec->table;
@@ -288,8 +290,9 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
         const bool level1_only = BATCH && (P.launch_steps == 1 || rec->stop - clock == 1);
 
         auto at = [&](const T *base, int f, int xx, int yy) { return base + f * FE + yy * BX + xx; };
-        auto coef = [&](uint32_t ip, int which, float4 &a, float4 &b) {   // which: 0 ce, 1 ch
-            if (id_mode && !(which && ch_uni)) {
+        // which: 0 ce, 1 ch; ids: whether the tile looks its coefficients up by id
+        auto coef = [&](uint32_t ip, int which, float4 &a, float4 &b, bool ids) {
+            if (ids && !(which && ch_uni)) {
                 a = stab[2 * (ip & 0xff) + which];
                 b = stab[2 * (ip >> 8) + which];
             } else {
@@ -315,11 +318,16 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
             return v;
         };
 
-        // One z-plane iteration.  ST (steady): k in [ks, kz1), where every phase runs, no mask depends on
+        // One z-plane iteration.  steady 0: any plane.  ST (steady 1, and in a batch 1 for a tile with PEC-coded
+        // ids and 2 for one of a uniform cavity): k in [ks, kz1), where every phase runs, no mask depends on
         // k, and a failed ring wait only drops the stores: the phases then read a stale slot (in bounds)
         // instead of being skipped, so nothing is zeroed or voted per plane.
         auto plane_step = [&](const int k, auto steady) {
-            constexpr bool ST = decltype(steady)::value;
+            constexpr int KIND = decltype(steady)::value;
+            constexpr bool ST = KIND != 0;
+            constexpr bool NOMASK = ST && (BATCH ? KIND == 1 : PEC_TABLE);
+            const bool ids = BATCH && ST ? KIND == 1 : id_mode;
+            const bool level1 = BATCH && ST ? false : level1_only;   // one-step tiles take no steady planes
             int sb = sa + 1;
             uint32_t pb = pa;
             if (sb == S) {
@@ -335,8 +343,8 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
             const uint8_t *ida = slots + sa * SB + IDO;
             // H2(k-1) needs plane k-1 >= 0 (its inputs at plane -1 were never written)
             const bool do_e1 = ST || k >= kz0 - 1;
-            const bool do_h2 = !level1_only && (ST || (k >= kz0 && k >= 1));
-            const bool do_e2 = !level1_only && (ST || k >= kz0 + 1);
+            const bool do_h2 = !level1 && (ST || (k >= kz0 && k >= 1));
+            const bool do_e2 = !level1 && (ST || k >= kz0 + 1);
             float *e1cur = e1b + (k & 1) * 2 * PF, *e1prv = e1b + ((k + 1) & 1) * 2 * PF;
 
             // ---------------- phase 1: H1(k) on the lane's two cells
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 h1y_ = Pair<T>::ld(at(A, 4, bx, by));
                 h1z_ = Pair<T>::ld(at(A, 5, bx, by));
                 // idoff is even (x0 and the 16-byte id box origin are), so the lane's two ids are one aligned u16
-                if (id_mode) idpair = *reinterpret_cast<const uint16_t *>(ida + by * G::IBX + idoff + 2 * lane);
+                if (ids) idpair = *reinterpret_cast<const uint16_t *>(ida + by * G::IBX + idoff + 2 * lane);
                 float4 ca, cb;
                 if (FULL_H) {
                     const float2 cx = cload(slots + sa * SB, 3), cy = cload(slots + sa * SB, 4), cz = cload(slots + sa * SB, 5);
@@ -367,7 +375,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                     chn_y = cy;
                     chn_z = cz;
                 } else {
-                    coef(idpair, 1, ca, cb);
+                    coef(idpair, 1, ca, cb, ids);
                 }
                 const float2 ez_x1 = make_float2(e0z.y, ez_x2), ey_x1 = make_float2(e0y.y, ey_x2);
                 h1x_ = fma2(make_float2(ca.x, cb.x), sub2(sub2(eyb, e0y), sub2(ez_y1, e0z)), h1x_);
@@ -393,12 +401,11 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                     ca = make_float4(cx.x, cy.x, cz.x, 0.f);
                     cb = make_float4(cx.y, cy.y, cz.y, 0.f);
                 } else {
-                    coef(idpair, 0, ca, cb);
+                    coef(idpair, 0, ca, cb, ids);
                 }
                 const bool inz = ST || k < nz, k1 = ST || k >= 1, j1 = gj >= 1;
                 const bool va = rowin && ina && inz, vb = rowin && inb && inz;
                 const bool i1a = gi >= 1;
-                constexpr bool NOMASK = ST && PEC_TABLE;
                 const float2 cex = NOMASK ? make_float2(ca.x, cb.x)
                                           : make_float2((j1 && k1) ? ca.x : 0.f, (j1 && k1) ? cb.x : 0.f);
                 const float2 cey = NOMASK ? make_float2(ca.y, cb.y)
@@ -416,7 +423,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 *reinterpret_cast<float2 *>(e1cur + pr * PW + pc) = e1x;
                 *reinterpret_cast<float2 *>(e1cur + PF + pr * PW + pc) = e1z;
                 // one step: (H1, E1) is the result
-                if (level1_only && ok && out_row && out_a && (ST || (k >= kz0 && k < kz1))) {
+                if (level1 && ok && out_row && out_a && (ST || (k >= kz0 && k < kz1))) {
                     const long long g = (long long)k * plane + (long long)gj * pitch + gi;
                     if (store_ok(P.status, g, 2, plane * nz)) {
                         Pair<T>::st_cs(dst0 + g, e1x.x, e1x.y);
@@ -446,7 +453,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                     ca = make_float4(chpx.x, chpy.x, chpz.x, 0.f);
                     cb = make_float4(chpx.y, chpy.y, chpz.y, 0.f);
                 } else {
-                    coef(idprev, 1, ca, cb);
+                    coef(idprev, 1, ca, cb, ids);
                 }
                 const float2 ez_x1 = make_float2(e1pz.y, ez_x2), ey_x1 = make_float2(e1py.y, ey_x2);
                 h2x = fma2(make_float2(ca.x, cb.x), sub2(sub2(e1y, e1py), sub2(ez_y1, e1pz)), h1px);
@@ -465,10 +472,9 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
                 const float2 hx_ym = *reinterpret_cast<const float2 *>(sh2x + (pr - 1) * PW + pc);
                 const float2 hz_ym = *reinterpret_cast<const float2 *>(sh2z + (pr - 1) * PW + pc);
                 float4 ca, cb;
-                if (!FULLC) coef(idprev, 0, ca, cb);
+                if (!FULLC) coef(idprev, 0, ca, cb, ids);
                 const int kk = k - 1;
                 const bool k1 = ST || kk >= 1, j1 = gj >= 1, i1a = gi >= 1;
-                constexpr bool NOMASK = ST && PEC_TABLE;
                 const float2 cex = FULLC ? cepx : NOMASK ? make_float2(ca.x, cb.x)
                                           : make_float2((j1 && k1) ? ca.x : 0.f, (j1 && k1) ? cb.x : 0.f);
                 const float2 cey = FULLC ? cepy : NOMASK ? make_float2(ca.y, cb.y)
@@ -523,16 +529,34 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
             }
         };
 
-        if (!SPLIT) {
+        using Any = std::integral_constant<int, 0>;
+        using Steady = std::integral_constant<int, 1>;
+        if (BSTEADY) {
+            using SteadyUniform = std::integral_constant<int, 2>;
+            // ids without PEC coding (more than 31 materials) and one-step tiles take the general body throughout
+            const int kind = level1_only ? 0 : rec->mode == COEF_SCALAR ? 2 : rec->pec ? 1 : 0;
+            for (int k = kb; k <= kz1;) {
+                if (kind == 1 && k >= ks && k < kz1) {
+#pragma unroll 2
+                    for (; k < kz1; ++k) plane_step(k, Steady{});
+                } else if (kind == 2 && k >= ks && k < kz1) {
+#pragma unroll 2
+                    for (; k < kz1; ++k) plane_step(k, SteadyUniform{});
+                } else {
+                    plane_step(k, Any{});
+                    ++k;
+                }
+            }
+        } else if (!SPLIT) {
 #pragma unroll 2   // consecutive planes renamed instead of copied (the carried z neighbours)
-            for (int k = kb; k <= kz1; ++k) plane_step(k, std::false_type{});
+            for (int k = kb; k <= kz1; ++k) plane_step(k, Any{});
         } else {
             for (int k = kb; k <= kz1;) {
                 if (k >= ks && k < kz1) {
 #pragma unroll 2
-                    for (; k < kz1; ++k) plane_step(k, std::true_type{});
+                    for (; k < kz1; ++k) plane_step(k, Steady{});
                 } else {
-                    plane_step(k, std::false_type{});
+                    plane_step(k, Any{});
                     ++k;
                 }
             }
@@ -604,6 +628,13 @@ int fused2_full_smem_bytes(int storage, int coef_class, int stages) {
                         : smem2_bytes<__half, kFullTileY, COEF_CLASS_FULL_UNIFORM_H>(stages);
 }
 
+// A batch with steady-state bodies (tile heights 8 and 12).
+template <int TY> static cudaError_t launch2_batch_steady(int storage, const FusedLaunch &L, cudaStream_t s) {
+    if (storage == 0) return launch2_typed<float, TY, true, COEF_CLASS_ANY_STEADY>(L, s);
+    if (storage == 1) return launch2_typed<__half, TY, true, COEF_CLASS_ANY_STEADY>(L, s);
+    return launch2_typed<__nv_bfloat16, TY, true, COEF_CLASS_ANY_STEADY>(L, s);
+}
+
 template <int CM> static cudaError_t launch2_full(int storage, const FusedLaunch &L, cudaStream_t s) {
     if (L.tile_y != kFullTileY) return cudaErrorInvalidValue;
     if (storage == 0) return launch2_typed<float, kFullTileY, false, CM>(L, s);
@@ -624,6 +655,8 @@ cudaError_t launch_fused2_step(int storage, const FusedLaunch &L, cudaStream_t s
     cudaError_t e = cudaErrorInvalidValue;
     if (L.coef_class == COEF_CLASS_FULL) return launch2_full<COEF_CLASS_FULL>(storage, L, s);
     if (L.coef_class == COEF_CLASS_FULL_UNIFORM_H) return launch2_full<COEF_CLASS_FULL_UNIFORM_H>(storage, L, s);
+    if (L.coef_class == COEF_CLASS_ANY_STEADY && L.tile_y == 12) return launch2_batch_steady<12>(storage, L, s);
+    if (L.coef_class == COEF_CLASS_ANY_STEADY && L.tile_y == 8) return launch2_batch_steady<8>(storage, L, s);
     if (L.step || L.launch_steps == 1)   // a batch launch (or a one-step store launch)
         FDTD_DISPATCH2(storage, L.tile_y, e = (launch2_typed<T, TY, true, COEF_CLASS_ANY>(L, s)));
     else if (L.coef_class == COEF_CLASS_SCALAR)

@@ -44,7 +44,7 @@ struct FusedLaunch {
                                // (NULL: CTA b takes tiles b, b + grid, b + 2 grid, ...)
     int launch_steps;          // two-step kernel: 2, or 1 (every tile stores its level-1 result only)
     int rows_per_warp;         // two-step kernel: 1 (k_fused2.cu) or 2 (k_fused2r.cu); 0 means 1
-    int coef_class;            // CoefClass shared by every tile (COEF_CLASS_ANY: read from each record)
+    int coef_class;            // CoefClass shared by every tile (COEF_CLASS_ANY*: read from each record)
 };
 // Coefficient layout shared by all tiles of a launch, so that a kernel can be compiled for it.
 enum CoefClass : int {
@@ -58,6 +58,7 @@ enum CoefClass : int {
     // COEF_FULL: per-position FP32 ce arrays (and ch arrays) streamed with the fields
     COEF_CLASS_FULL_UNIFORM_H = 6,
     COEF_CLASS_FULL = 7,
+    COEF_CLASS_ANY_STEADY = 8,    // a batch's tiles may differ, and most are deep enough for a steady-state body per layout
 };
 inline int coef_class_of(int coef_mode, int ch_uniform, bool pec_ids) {
     if (coef_mode == COEF_SCALAR) return COEF_CLASS_SCALAR;

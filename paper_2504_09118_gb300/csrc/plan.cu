@@ -174,6 +174,7 @@ TileRec base_rec(const fdtd_ctx *c, int parity_off, int set) {
     const bool pec = set == 1 && c->id_pec;
     r.table = reinterpret_cast<const float4 *>(pec ? c->table_pec : c->table_fused);
     r.ntab = pec ? c->ntab_pec : c->ntab;
+    r.pec = pec ? 1 : 0;
     if (set == 4) {   // per-position coefficients are stored unscaled: the kernel applies the ratios
         r.ce[0] = re;
         r.ce[1] = 1.0f / re;
