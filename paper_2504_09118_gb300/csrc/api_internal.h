@@ -120,7 +120,8 @@ struct fdtd_ctx {
     void *d_resident = nullptr;
     int order = 2;                          // spatial order of the differences (2: Eq. 2, 4: the (2,4) scheme)
     double courant = 0.0;                   // max over cells of 3 ce ch (stable for order 2 when <= 1)
-    int ch_uniform = 1;
+    int ch_uniform = 1;                     // per component the same ch in every cell (ch_s)
+    bool ch_const = true;                   // one ch for all components, far faces included (ch_s[0])
     fdtd_tuning tuning{};
     std::map<fdtd::GraphKey, cudaGraphExec_t> graphs;
     int inject_us = 0;

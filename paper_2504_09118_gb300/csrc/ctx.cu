@@ -82,6 +82,7 @@ CavityDesc make_desc(const fdtd_ctx *c, int parity_off) {
     d.kr_lo = 0;
     d.kr_hi = c->nz;
     d.face_top = 1;
+    d.ch_const = c->ch_const ? 1 : 0;
     return d;
 }
 
@@ -508,6 +509,7 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
                 else if (q == 1) src = cidx((int)(n % nx), ny, (int)(n / nx));
                 else src = cidx((int)(n % nx), (int)(n / nx), nz);
                 fc[n] = have_ch ? ch[q][src] : vac;
+                if (have_ch && fc[n] != ch[0][0]) c->ch_const = false;
             }
             if ((e = dmalloc(c, (void **)&c->face_ch[q], nface[q] * 4)) != cudaSuccess) return cfail("face alloc", e);
             if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cfail("sync", e);
@@ -612,6 +614,9 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
             }
         }
     }
+    // the interior: ch_uniform per component, and the three components alike (the far faces were compared above)
+    if (have_ch && !(c->ch_uniform && c->ch_s[0] == ch[0][0] && c->ch_s[1] == c->ch_s[0] && c->ch_s[2] == c->ch_s[0]))
+        c->ch_const = false;
     if ((e = dmalloc(c, (void **)&c->d_status, sizeof(int))) != cudaSuccess) return cfail("status alloc", e);
     if ((e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream)) != cudaSuccess) return cfail("memset", e);
     const int nb = reduction_blocks();

@@ -105,5 +105,95 @@ struct Acc {
     }
 };
 
+// ---------------------------------------------------------------------------------------------
+// The same on the two cells of a lane in packed FP32x2 instructions (one rounding per element, as the
+// scalar forms).  Values that a lane holds as aligned pairs need no register moves, so the compensated
+// chains cost half the issue slots, and the two cells' chains are independent.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e) {
+    const float2 t = add2(a, b), bb = sub2(t, a);
+    e = add2(sub2(a, sub2(t, bb)), sub2(b, bb));
+    s = t;
+}
+// a - b = s + e exactly.
+__device__ __forceinline__ void two_diff2(float2 a, float2 b, float2 &s, float2 &e) {
+    const float2 t = sub2(a, b), bb = sub2(t, a);
+    e = sub2(sub2(a, sub2(t, bb)), add2(b, bb));
+    s = t;
+}
+__device__ __forceinline__ void two_prod2(float2 a, float2 b, float2 &p, float2 &e) {
+    const float2 t = mul2(a, b);
+    e = fma2(a, b, neg2(t));
+    p = t;
+}
+
+// Two values held as unevaluated sums.
+struct F22 {
+    float2 hi, lo;
+};
+
+// (a - b) - (c - d) as a pair.
+__device__ __forceinline__ F22 diff22(float2 a, float2 b, float2 c, float2 d) {
+    float2 x, ex, y, ey, s, es;
+    two_diff2(a, b, x, ex);
+    two_diff2(c, d, y, ey);
+    two_diff2(x, y, s, es);
+    return F22{s, add2(es, sub2(ex, ey))};
+}
+
+// Two Dot2 accumulators.
+struct Acc2 {
+    float2 p = make_float2(0.f, 0.f), s = make_float2(0.f, 0.f);
+    __device__ __forceinline__ void prod(float2 x, float2 y) {
+        float2 h, r, q;
+        two_prod2(x, y, h, r);
+        two_sum2(p, h, p, q);
+        s = add2(s, add2(q, r));
+    }
+    __device__ __forceinline__ void prod(float2 x, F22 y) {
+        prod(x, y.hi);
+        s = fma2(x, y.lo, s);
+    }
+    __device__ __forceinline__ void sq_times(float2 x, F22 c) {
+        float2 p2, e2;
+        two_prod2(x, x, p2, e2);
+        prod(p2, c.hi);
+        s = add2(s, fma2(p2, c.lo, mul2(e2, c.hi)));
+    }
+    // += (v.hi + v.lo)^2 (the lo^2 term is 2^-48 below and dropped)
+    __device__ __forceinline__ void square(F22 v) {
+        prod(v.hi, v.hi);
+        s = fma2(add2(v.hi, v.hi), v.lo, s);
+    }
+    __device__ __forceinline__ F22 pair() const {
+        F22 r;
+        two_sum2(p, s, r.hi, r.lo);
+        return r;
+    }
+    // the sum of both accumulators as a pair, and a fresh start
+    __device__ __forceinline__ F2 take() {
+        F2 r;
+        float e;
+        two_sum(p.x, p.y, r.hi, e);
+        r.lo = __fadd_rn(e, __fadd_rn(s.x, s.y));
+        p = s = make_float2(0.f, 0.f);
+        return r;
+    }
+};
+
+// a + b of pairs.
+__device__ __forceinline__ F2 add(F2 a, F2 b) {
+    F2 r;
+    float e;
+    two_sum(a.hi, b.hi, r.hi, e);
+    r.lo = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
+    return r;
+}
+
 }  // namespace df
 }  // namespace fdtd

@@ -75,7 +75,8 @@ struct CavityDesc {
     float inv_ce[3], inv_ch[3];  // COEF_SCALAR reciprocals
     // Reductions sum over the cells of planes [kr_lo, kr_hi) (the owned cells of a z-slab; the whole
     // cavity otherwise) and include the far face k = nz when face_top is set.
-    int kr_lo, kr_hi, face_top, pad1;
+    int kr_lo, kr_hi, face_top;
+    int ch_const;           // one ch (ch[0]) at every H position, far faces included
 };
 
 // Physical (unscaled) value of field f at linear offset off of copy `copy`.

@@ -263,7 +263,9 @@ __global__ void simple_e_kernel(const CavityDesc d, int copy) {
 }
 
 constexpr int kRedThreads = 256;
-constexpr int kRedBlocks = 1216;   // 8 x 152 SMs; fixed so that the summation order is reproducible
+constexpr int kRedBlocks = 1216;     // partials allocated: 8 x 152 SMs, the fourth-order reductions' grid
+constexpr int kRedPerSM = 3;                 // blocks per SM of the second-order reductions (their registers allow no more):
+constexpr int kRed2Blocks = 152 * kRedPerSM;   // one wave; grids are fixed so that the summation order is reproducible
 
 __device__ __forceinline__ double block_sum(double v, double *sh) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -277,37 +279,6 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return r;
 }
 
-// Reciprocal coefficients of the reductions as pairs (df.cuh): 1/ce (c = 0..2) and 1/ch (c = 3..5).
-// Material-id mode keeps them in a shared table (filled by the block before use), scalar mode in six
-// registers; per-position arrays take the reciprocal per cell (that mode is rare and slow anyway).
-struct InvCoefDF {
-    const CavityDesc *d;
-    const df::F2 *tab;   // shared, 6 per id (COEF_ID8)
-    df::F2 sc[6];        // COEF_SCALAR
-    __device__ __forceinline__ df::F2 operator()(int c, long long o, int m) const {
-        if (d->coef_mode == COEF_ID8) return tab[6 * m + c];
-        if (d->coef_mode == COEF_SCALAR) return sc[c];
-        return df::recip(d->coef[c][o]);
-    }
-};
-
-// Fills tab (6 * ntab pairs, shared) and the scalar reciprocals; call with the whole block, then sync.
-__device__ __forceinline__ InvCoefDF make_inv_coef_df(const CavityDesc &d, df::F2 *tab) {
-    InvCoefDF r;
-    r.d = &d;
-    r.tab = tab;
-    for (int c = 0; c < 3; ++c) {
-        r.sc[c] = df::recip(d.ce[c]);
-        r.sc[3 + c] = df::recip(d.ch[c]);
-    }
-    if (d.coef_mode == COEF_ID8)
-        for (int e = threadIdx.x; e < 6 * d.ntab; e += blockDim.x) {
-            const int m = e / 6, c = e % 6;
-            tab[e] = df::recip(d.table[8 * m + (c < 3 ? c : c + 1)]);
-        }
-    return r;
-}
-
 // 1/ch at far-face entry fi of face array c, as a pair and in FP64.
 __device__ __forceinline__ df::F2 face_inv_ch_df(const CavityDesc &d, int c, long long fi) {
     return df::recip(d.coef_mode == COEF_SCALAR ? d.ch[c] : d.face_ch[c][fi]);
@@ -316,79 +287,193 @@ __device__ __forceinline__ double face_inv_ch64(const CavityDesc &d, int c, long
     return d.coef_mode == COEF_SCALAR ? 1.0 / (double)d.ch[c] : 1.0 / (double)d.face_ch[c][fi];
 }
 
-// Per block, in a fixed order (warps over rows, lanes along x; far-face H appended):
+// Two adjacent values of field f from an even x index (rows are 128-byte aligned; past an odd nx lies padding).
+template <typename T> __device__ __forceinline__ float2 ld_pair(const CavityDesc &d, int copy, int f, long long off) {
+    const T *p = static_cast<const T *>(d.buf[copy][f]) + off;
+    float2 v;
+    if constexpr (Storage<T>::kind == 0) v = *reinterpret_cast<const float2 *>(p);
+    else if constexpr (Storage<T>::kind == 1) v = __half22float2(*reinterpret_cast<const __half2 *>(p));
+    else v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+    if (Storage<T>::scaled) {
+        v.x *= d.inv_scale[f];
+        v.y *= d.inv_scale[f];
+    }
+    return v;
+}
+
+// Per block, in a fixed order (a warp per (j, k) row, a lane two adjacent cells; far-face H appended):
 //   WHAT == 0: energy sum  E^2/ce + H^2/ch - H curl E   (W without the 1/2 dt/dx factor)
 //   WHAT == 1: sum of divE^2 over interior nodes and of divH^2 over cells.
-// Every term is formed from the stored values with error-free FP32 transformations (the curl
-// differences as exact pairs, the reciprocal coefficients as pairs; df.cuh) and a lane accumulates
-// its cells of a row with Dot2, about 2^-48 relative; the row sums are added in FP64, then per block
-// and over blocks in a fixed order, so the result is deterministic.  (GB300's FP64 rate made the same
-// sums in FP64 eight times slower at 512^3.)
-template <typename T, int WHAT>
-__global__ void __launch_bounds__(kRedThreads) reduce_kernel(const CavityDesc d, int copy, double *partial) {
+// Every term is formed from the stored values with error-free FP32 transformations (the curl differences
+// as exact pairs, the reciprocal coefficients as pairs; df.cuh) and a lane accumulates its cells of a row
+// with Dot2, about 2^-48 relative; the row sums are added in FP64, then per block and over blocks in a fixed
+// order, so the result is deterministic.  (GB300's FP64 rate made the same sums in FP64 eight times slower
+// at 512^3.)  CHC: one ch everywhere, far faces included: H^2 takes no lookups, and divH is an exact sum of six
+// values, scaled once.
+// Bound by the compensated FP32 arithmetic and the latency of the loads that 24 warps per SM (80 registers) leave:
+// packed pairs and separate accumulator chains against one cell and one chain per lane took the energy of 320^3
+// FP32 cells from 369 to 300 us and the divergences from 645 to 386 us (a DRAM pass over the state is 121 us).
+// Two blocks per SM (99-120 registers) 306 and 500 us; an L2 prefetch of the warp's next row: no gain.
+template <typename T, int WHAT, bool CHC>
+__global__ void __launch_bounds__(kRedThreads, kRedPerSM) reduce_kernel(const CavityDesc d, int copy, double *partial) {
     __shared__ double sh[kRedThreads / 32];
-    __shared__ df::F2 itab[6 * kMaxTable];
-    const int nx = d.nx, ny = d.ny;
+    __shared__ float thi[6 * kMaxTable], tlo[6 * kMaxTable];   // 1/ce xyz, 1/ch xyz by material id, as pairs
+    const int nx = d.nx, ny = d.ny, nz = d.nz;
     const long long P = d.pitch, Z = d.plane;
     double s0 = 0.0, s1 = 0.0;
-    const bool ids = d.coef_mode == COEF_ID8;
-    const InvCoefDF IC = make_inv_coef_df(d, itab);
+    const bool ids = d.coef_mode == COEF_ID8, scalar = d.coef_mode == COEF_SCALAR;
+    // a uniform cavity is one entry of the table (read at index 0 by every lane)
+    const int ntab = ids ? d.ntab : scalar ? 1 : 0;
+    for (int e = threadIdx.x; e < 6 * ntab; e += blockDim.x) {
+        const int c = e / ntab, m = e - c * ntab;
+        const df::F2 r = df::recip(scalar ? (c < 3 ? d.ce[c] : d.ch[c - 3]) : d.table[8 * m + (c < 3 ? c : c + 1)]);
+        thi[c * kMaxTable + m] = r.hi;
+        tlo[c * kMaxTable + m] = r.lo;
+    }
+    const df::F2 ich = df::recip(d.ch[0]);   // CHC
+    const df::F22 ich2{make_float2(ich.hi, ich.hi), make_float2(ich.lo, ich.lo)};
     __syncthreads();
-    const int nz = d.nz;
-    auto F = [&](int f, long long o) -> float { return ld_field<T>(d, copy, f, o); };
-    auto ICo = [&](int c, long long o) -> df::F2 { return IC(c, o, ids ? d.id[o] : 0); };
-    // one warp per (j, k) row, lanes along x: coalesced loads
+    const float2 zero = make_float2(0.f, 0.f);
+    // material ids of the two cells at off (packed), and 1/ce or 1/ch (c) of them
+    auto IDS = [&](long long off) -> unsigned { return ids ? *reinterpret_cast<const uint16_t *>(d.id + off) : 0u; };
+    bool two = true;   // the pair's second cell lies in the cavity (past an odd nx coefficient arrays hold 0)
+    auto IC = [&](int c, unsigned m, long long off) -> df::F22 {
+        if (d.coef_mode == COEF_FULL) {
+            const df::F2 a = df::recip(d.coef[c][off]), b = two ? df::recip(d.coef[c][off + 1]) : a;
+            return df::F22{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)};
+        }
+        const float *h = thi + c * kMaxTable, *l = tlo + c * kMaxTable;
+        return df::F22{make_float2(h[m & 0xff], h[m >> 8]), make_float2(l[m & 0xff], l[m >> 8])};
+    };
     const int lane = threadIdx.x & 31;
     // rows of the planes [kr_lo, kr_hi) (the owned cells of a z-slab; every plane otherwise)
-    const long long nrows = (long long)ny * (d.kr_hi - d.kr_lo);
-    const long long nwarps = ((long long)gridDim.x * kRedThreads) >> 5;
-    for (long long r = ((long long)blockIdx.x * kRedThreads + threadIdx.x) >> 5; r < nrows; r += nwarps) {
-        const int j = (int)(r % ny), k = d.kr_lo + (int)(r / ny);
-        df::Acc a0, a1;
-        for (int i = lane; i < nx; i += 32) {
+    // (at most 32768^2 of them: 32 bits; a 64-bit division per row showed)
+    const unsigned nrows = (unsigned)ny * (unsigned)(d.kr_hi - d.kr_lo);
+    const unsigned nwarps = (gridDim.x * kRedThreads) >> 5;
+    for (unsigned r = (blockIdx.x * kRedThreads + threadIdx.x) >> 5; r < nrows; r += nwarps) {
+        const unsigned kr = r / (unsigned)ny;
+        const int j = (int)(r - kr * (unsigned)ny), k = d.kr_lo + (int)kr;
+        df::Acc2 a0, a1, a2;
+        for (int i = 2 * lane; i < nx; i += 64) {
             const long long o = (long long)k * Z + (long long)j * P + i;
-            const float ex = F(0, o), ey = F(1, o), ez = F(2, o), hx = F(3, o), hy = F(4, o), hz = F(5, o);
-            const int m = ids ? d.id[o] : 0;
+            two = i + 1 < nx;
+            auto F = [&](int f, long long off) -> float2 {
+                float2 v = ld_pair<T>(d, copy, f, off);
+                if (!two) v.y = 0.f;
+                return v;
+            };
+            // the pair one cell up in x: (v.y, the cell after)
+            auto up = [&](int f, float2 v) -> float2 {
+                return make_float2(v.y, i + 2 < nx ? ld_field<T>(d, copy, f, o + 2) : 0.f);
+            };
+            const float2 ex = F(0, o), ey = F(1, o), ez = F(2, o), hx = F(3, o), hy = F(4, o), hz = F(5, o);
+            const unsigned m = IDS(o);
             if (WHAT == 0) {
-                const float ex_j1 = j + 1 < ny ? F(0, o + P) : 0.f, ex_k1 = k + 1 < nz ? F(0, o + Z) : 0.f;
-                const float ey_i1 = i + 1 < nx ? F(1, o + 1) : 0.f, ey_k1 = k + 1 < nz ? F(1, o + Z) : 0.f;
-                const float ez_i1 = i + 1 < nx ? F(2, o + 1) : 0.f, ez_j1 = j + 1 < ny ? F(2, o + P) : 0.f;
-                a0.sq_times(ex, IC(0, o, m));
-                a0.sq_times(ey, IC(1, o, m));
-                a0.sq_times(ez, IC(2, o, m));
-                a0.sq_times(hx, IC(3, o, m));
-                a0.prod(-hx, df::diff2(ez_j1, ez, ey_k1, ey));
-                a0.sq_times(hy, IC(4, o, m));
-                a0.prod(-hy, df::diff2(ex_k1, ex, ez_i1, ez));
-                a0.sq_times(hz, IC(5, o, m));
-                a0.prod(-hz, df::diff2(ey_i1, ey, ex_j1, ex));
+                const float2 ex_j1 = j + 1 < ny ? F(0, o + P) : zero, ez_j1 = j + 1 < ny ? F(2, o + P) : zero;
+                const float2 ex_k1 = k + 1 < nz ? F(0, o + Z) : zero, ey_k1 = k + 1 < nz ? F(1, o + Z) : zero;
+                const float2 ey_i1 = up(1, ey), ez_i1 = up(2, ez);
+                a0.sq_times(ex, IC(0, m, o));
+                a0.sq_times(ey, IC(1, m, o));
+                a0.sq_times(ez, IC(2, m, o));
+                // (H^2 summed first and scaled once is cheaper and 1.5 times less exact: the unscaled squares of
+                // short-mantissa values round with a bias)
+                a1.sq_times(hx, CHC ? ich2 : IC(3, m, o));
+                a1.sq_times(hy, CHC ? ich2 : IC(4, m, o));
+                a1.sq_times(hz, CHC ? ich2 : IC(5, m, o));
+                // past an odd nx the second cell's H is 0, so its curl does not count
+                a2.prod(hx, df::diff22(ez_j1, ez, ey_k1, ey));
+                a2.prod(hy, df::diff22(ex_k1, ex, ez_i1, ez));
+                a2.prod(hz, df::diff22(ey_i1, ey, ex_j1, ex));
             } else {
-                if (i >= 1 && j >= 1 && k >= 1) {
-                    df::Acc de;   // sum over c of D_c(node) - D_c(node - e_c), D = E / ce
-                    de.prod(ex, IC(0, o, m));
-                    de.prod(-F(0, o - 1), ICo(0, o - 1));
-                    de.prod(ey, IC(1, o, m));
-                    de.prod(-F(1, o - P), ICo(1, o - P));
-                    de.prod(ez, IC(2, o, m));
-                    de.prod(-F(2, o - Z), ICo(2, o - Z));
-                    a0.square(de.pair());
+                if (j >= 1 && k >= 1) {
+                    df::Acc2 de;   // sum over c of D_c(node) - D_c(node - e_c), D = E / ce
+                    df::F22 cx = IC(0, m, o), cl;
+                    float2 exl;    // the pair one cell down in x
+                    exl.y = ex.x;
+                    cl.hi.y = cx.hi.x;
+                    cl.lo.y = cx.lo.x;
+                    if (i > 0) {
+                        exl.x = ld_field<T>(d, copy, 0, o - 1);
+                        if (d.coef_mode == COEF_FULL) {
+                            const df::F2 q = df::recip(d.coef[0][o - 1]);
+                            cl.hi.x = q.hi;
+                            cl.lo.x = q.lo;
+                        } else {
+                            const int q = ids ? d.id[o - 1] : 0;
+                            cl.hi.x = thi[q];
+                            cl.lo.x = tlo[q];
+                        }
+                    } else {
+                        exl.x = cl.hi.x = cl.lo.x = 0.f;
+                    }
+                    de.prod(ex, cx);
+                    de.prod(df::neg2(exl), cl);
+                    de.prod(ey, IC(1, m, o));
+                    de.prod(df::neg2(F(1, o - P)), IC(1, IDS(o - P), o - P));
+                    de.prod(ez, IC(2, m, o));
+                    de.prod(df::neg2(F(2, o - Z)), IC(2, IDS(o - Z), o - Z));
+                    df::F22 v = de.pair();
+                    if (i == 0) v.hi.x = v.lo.x = 0.f;       // not a node inside
+                    if (!two) v.hi.y = v.lo.y = 0.f;
+                    a0.square(v);
                 }
-                df::Acc dh;   // sum over c of B_c(cell + e_c) - B_c(cell), B = H / ch
+                // sum over c of B_c(cell + e_c) - B_c(cell), B = H / ch
                 const long long fx = (long long)k * ny + j, fy = (long long)k * nx + i, fz = (long long)j * nx + i;
-                if (i + 1 < nx) dh.prod(F(3, o + 1), ICo(3, o + 1));
-                else dh.prod(d.face[0][fx], face_inv_ch_df(d, 0, fx));
-                if (j + 1 < ny) dh.prod(F(4, o + P), ICo(4, o + P));
-                else dh.prod(d.face[1][fy], face_inv_ch_df(d, 1, fy));
-                if (k + 1 < nz) dh.prod(F(5, o + Z), ICo(5, o + Z));
-                else dh.prod(d.face[2][fz], face_inv_ch_df(d, 2, fz));
-                dh.prod(-hx, IC(3, o, m));
-                dh.prod(-hy, IC(4, o, m));
-                dh.prod(-hz, IC(5, o, m));
-                a1.square(dh.pair());
+                float2 hx1 = up(3, hx), hy1, hz1;
+                if (i + 1 >= nx) hx1.x = d.face[0][fx];
+                else if (i + 2 >= nx) hx1.y = d.face[0][fx];
+                auto face2 = [&](const float *f, long long at) { return make_float2(f[at], two ? f[at + 1] : 0.f); };
+                hy1 = j + 1 < ny ? F(4, o + P) : face2(d.face[1], fy);
+                hz1 = k + 1 < nz ? F(5, o + Z) : face2(d.face[2], fz);
+                if (CHC) {   // the difference as an exact sum; 1/ch^2 scales the total
+                    float2 x, exx, y, eyy, z, ezz, t, et, u, eu;
+                    df::two_diff2(hx1, hx, x, exx);
+                    df::two_diff2(hy1, hy, y, eyy);
+                    df::two_diff2(hz1, hz, z, ezz);
+                    df::two_sum2(x, y, t, et);
+                    df::two_sum2(t, z, u, eu);
+                    df::F22 v{u, df::add2(df::add2(df::add2(exx, eyy), df::add2(ezz, et)), eu)};
+                    if (!two) v.hi.y = v.lo.y = 0.f;
+                    a1.square(v);
+                } else {
+                    df::F22 c;
+                    auto set = [](df::F22 &f, int e, df::F2 v) {
+                        if (e == 0) { f.hi.x = v.hi; f.lo.x = v.lo; }
+                        else { f.hi.y = v.hi; f.lo.y = v.lo; }
+                    };
+                    auto one = [&](int q, long long off) -> df::F2 {   // 1/ch component q at one cell
+                        if (d.coef_mode == COEF_FULL) return df::recip(d.coef[3 + q][off]);
+                        const int n = ids ? d.id[off] : 0;
+                        return df::F2{thi[(3 + q) * kMaxTable + n], tlo[(3 + q) * kMaxTable + n]};
+                    };
+                    df::Acc2 dh;
+                    set(c, 0, i + 1 < nx ? one(0, o + 1) : face_inv_ch_df(d, 0, fx));
+                    set(c, 1, i + 2 < nx ? one(0, o + 2) : face_inv_ch_df(d, 0, fx));
+                    dh.prod(hx1, c);
+                    if (j + 1 < ny) c = IC(4, IDS(o + P), o + P);
+                    else for (int e = 0; e < 2; ++e) set(c, e, face_inv_ch_df(d, 1, two ? fy + e : fy));
+                    dh.prod(hy1, c);
+                    if (k + 1 < nz) c = IC(5, IDS(o + Z), o + Z);
+                    else for (int e = 0; e < 2; ++e) set(c, e, face_inv_ch_df(d, 2, two ? fz + e : fz));
+                    dh.prod(hz1, c);
+                    dh.prod(df::neg2(hx), IC(3, m, o));
+                    dh.prod(df::neg2(hy), IC(4, m, o));
+                    dh.prod(df::neg2(hz), IC(5, m, o));
+                    df::F22 v = dh.pair();
+                    if (!two) v.hi.y = v.lo.y = 0.f;
+                    a1.square(v);
+                }
             }
         }
-        s0 += a0.take();
-        s1 += a1.take();
+        // the row's sum in FP64 (one pair per row: FP64 additions are the scarce operation)
+        if (WHAT == 0) {
+            const df::F2 c = a2.take(), t = df::add(df::add(a0.take(), a1.take()), df::F2{-c.hi, -c.lo});
+            s0 += (double)t.hi + (double)t.lo;
+        } else {
+            const df::F2 e = a0.take(), h = a1.take();
+            s0 += (double)e.hi + (double)e.lo;
+            s1 += (double)h.hi + (double)h.lo;
+        }
     }
     if (WHAT == 0) {
         // constant far-face normal H: curl E vanishes there, so its energy term is H^2/ch (the x and y
@@ -403,8 +488,11 @@ __global__ void __launch_bounds__(kRedThreads) reduce_kernel(const CavityDesc d,
             else if (n < nfx + nfy) { c = 1; fi = n - nfx + (long long)d.kr_lo * nx; }
             else { c = 2; fi = n - nfx - nfy; }
             const double h = d.face[c][fi];
-            s0 += h * h * face_inv_ch64(d, c, fi);
+            s0 += h * h * (CHC ? 1.0 / (double)d.ch[0] : face_inv_ch64(d, c, fi));
         }
+    } else if (CHC) {
+        const double q = 1.0 / (double)d.ch[0];
+        s1 *= q * q;
     }
     const double a = block_sum(s0, sh);
     const double b = block_sum(s1, sh);
@@ -503,10 +591,17 @@ cudaError_t launch_reductions(int storage, const CavityDesc &d, int copy, int wh
     if (order == 4) {
         cudaError_t e = launch_reductions4(storage, d, copy, what, partial, nblocks, s);
         if (e != cudaSuccess) return e;
-    } else if (what == 0)
-        FDTD_STORAGE_DISPATCH(storage, reduce_kernel<T, 0><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial));
-    else
-        FDTD_STORAGE_DISPATCH(storage, reduce_kernel<T, 1><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial));
+    } else {
+        nblocks = kRed2Blocks;
+        if (what == 0 && d.ch_const)
+            FDTD_STORAGE_DISPATCH(storage, (reduce_kernel<T, 0, true><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial)));
+        else if (what == 0)
+            FDTD_STORAGE_DISPATCH(storage, (reduce_kernel<T, 0, false><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial)));
+        else if (d.ch_const)
+            FDTD_STORAGE_DISPATCH(storage, (reduce_kernel<T, 1, true><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial)));
+        else
+            FDTD_STORAGE_DISPATCH(storage, (reduce_kernel<T, 1, false><<<nblocks, kRedThreads, 0, s>>>(d, copy, partial)));
+    }
     reduce_final_kernel<<<1, kRedThreads, 0, s>>>(partial, nblocks, status, out);
     return cudaGetLastError();
 }
