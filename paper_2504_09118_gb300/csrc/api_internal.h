@@ -162,12 +162,13 @@ struct fdtd_batch {
     std::vector<Member> members;
     long long step = 0;              // step clock: steps enqueued so far (a two-step launch advances it by 2)
     long long launches = 0;          // launches enqueued so far; the next launch has parity launches & 1
-    long long *d_step = nullptr;     // device copy of the step clock (advanced by a kernel after each launch)
+    long long *d_step = nullptr;     // device copy of the step clock (moved by every launch, or a kernel after it), CTA count
     fdtd_tuning tuning{};
     TileRec *d_tiles = nullptr;      // tile records, then (at d_first) the per-CTA range offsets
     int *d_first = nullptr;          // grid + 1 offsets when the tiles are assigned to CTAs on the host, else NULL
     int tiles_cap = 0, ntiles = 0, grid = 0;
     Shape shape;                     // launch shape the tile list was built for
+    long long cells = 0;             // of the running members
     bool steady = false;             // two-step kernel: the instance with steady-state plane bodies
     // pinned staging of the tile-list uploads, two buffers used in turn: a copy from pageable memory may
     // wait for the stream, which would drain the queued launches at every change of membership

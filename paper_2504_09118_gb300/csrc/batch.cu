@@ -17,9 +17,9 @@ int fdtd_batch_create(fdtd_batch **out, int storage, void *cuda_stream) {
     b->storage = storage;
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     bool ok = pool_alloc((void **)&b->d_status, sizeof(int), b->stream) == cudaSuccess &&
-              pool_alloc((void **)&b->d_step, sizeof(long long), b->stream) == cudaSuccess &&
+              pool_alloc((void **)&b->d_step, 2 * sizeof(long long), b->stream) == cudaSuccess &&
               cudaMemsetAsync(b->d_status, 0, sizeof(int), b->stream) == cudaSuccess &&
-              cudaMemsetAsync(b->d_step, 0, sizeof(long long), b->stream) == cudaSuccess &&
+              cudaMemsetAsync(b->d_step, 0, 2 * sizeof(long long), b->stream) == cudaSuccess &&
               cudaEventCreateWithFlags(&b->done_ev, cudaEventDisableTiming) == cudaSuccess &&
               cudaStreamSynchronize(b->stream) == cudaSuccess;
     if (!ok) {
@@ -225,6 +225,7 @@ static int batch_rebuild(fdtd_batch *b) {
     long long stop0 = -1;
     std::vector<std::pair<int, long long>> columns;   // (nz, tile columns) of each running member
     int max_nz = 1;
+    long long cells = 0;
     for (auto &mb : b->members) {
         if (mb.stop <= b->step) continue;   // finished members carry no tiles
         fdtd_ctx *c = mb.c;
@@ -233,6 +234,7 @@ static int batch_rebuild(fdtd_batch *b) {
         total_cols += cols;
         total_cols_planes += cols * c->nz;
         columns.emplace_back(c->nz, cols);
+        cells += (long long)c->nx * c->ny * c->nz;
         max_nz = std::max(max_nz, c->nz);
         if (stop0 < 0) stop0 = mb.stop;
         same_stop = same_stop && mb.stop == stop0;
@@ -317,6 +319,7 @@ static int batch_rebuild(fdtd_batch *b) {
     b->ntiles = (int)tiles.size();
     b->grid = grid;
     b->shape = s;
+    b->cells = cells;
     b->steady = kind == 1 && s.rows_per_warp == 1 && s.tile_y <= 12;   // no instance with 16 rows
     b->dirty = false;
     return FDTD_OK;
@@ -338,11 +341,13 @@ static int batch_launch(fdtd_batch *b, int parity, int nsteps) {
     L.grid = b->grid;
     L.launch_steps = nsteps;
     L.rows_per_warp = s.rows_per_warp;
+    L.overlap = b->cells < kOverlapCells;
     L.coef_class = b->steady ? COEF_CLASS_ANY_STEADY : COEF_CLASS_ANY;
     cudaError_t e = kind == 0   ? launch_fused_step(b->storage, L, b->stream)
                     : kind == 1 ? launch_fused2_step(b->storage, L, b->stream)
                                 : launch_fused4_step(b->storage, L, b->stream);
-    if (e == cudaSuccess) e = launch_step_counter(b->d_step, nsteps, b->stream);
+    const bool own_clock = kind == 1 && s.rows_per_warp == 1 && L.ntiles > 0;   // the kernel moved the clock
+    if (e == cudaSuccess && !own_clock) e = launch_step_counter(b->d_step, nsteps, b->stream);
     if (e != cudaSuccess) return bfail(b, FDTD_ERR_CUDA, "batch launch: %s", cudaGetErrorString(e));
     return FDTD_OK;
 }

@@ -12,8 +12,19 @@ namespace fdtd {
 
 namespace {
 
+struct ExtrasArgs {
+    CavityDesc d;
+    ExtrasParams X;
+    int copy;
+};
+
 template <typename T>
-__global__ void extras_kernel(const CavityDesc d, int copy, const ExtrasParams X) {
+__global__ void extras_kernel(const ExtrasArgs A) {
+    const CavityDesc &d = A.d;
+    const ExtrasParams &X = A.X;
+    const int copy = A.copy;
+    grid_launch_dependents();
+    grid_wait_previous();
     const long long n = *X.clock;   // index of the step just taken (counted from fdtd_set_fields)
     if (threadIdx.x == 0)
         for (int s = 0; s < X.nsrc; ++s) {   // serial: several currents may share a position
@@ -35,14 +46,14 @@ __global__ void extras_kernel(const CavityDesc d, int copy, const ExtrasParams X
 
 }  // namespace
 
+template <typename T> static cudaError_t launch_extras_typed(const CavityDesc &d, int copy, const ExtrasParams &X, cudaStream_t s) {
+    return launch_overlapped(extras_kernel<T>, 1, 128, 0, s, ExtrasArgs{d, X, copy}, true);
+}
+
 cudaError_t launch_extras(int storage, const CavityDesc &d, int copy, const ExtrasParams &X, cudaStream_t s) {
-    if (storage == 0)
-        extras_kernel<float><<<1, 128, 0, s>>>(d, copy, X);
-    else if (storage == 1)
-        extras_kernel<__half><<<1, 128, 0, s>>>(d, copy, X);
-    else
-        extras_kernel<__nv_bfloat16><<<1, 128, 0, s>>>(d, copy, X);
-    return cudaGetLastError();
+    if (storage == 0) return launch_extras_typed<float>(d, copy, X, s);
+    if (storage == 1) return launch_extras_typed<__half>(d, copy, X, s);
+    return launch_extras_typed<__nv_bfloat16>(d, copy, X, s);
 }
 
 }  // namespace fdtd

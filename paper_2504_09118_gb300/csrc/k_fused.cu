@@ -154,9 +154,12 @@ __global__ void __launch_bounds__(block_threads<TY>(), (TY <= 8 ? 2 : 1)) fused_
         fence_proxy_async_smem();
     }
     __syncthreads();
+    if (!P.step) grid_launch_dependents();   // a single cavity (a batch's launches read the clock above)
 
     // =========================================================== producer warp
     if (warp == TY + 1) {
+        // everything before reads launch-constant records only; the consumers' stores follow data loaded after this
+        if (!P.step) grid_wait_previous();
         int issued = 0, m = 0;
         int s = 0;           // slot of the next unit
         uint32_t rnd = 0;    // parity of the ring round of the next unit
@@ -445,8 +448,7 @@ cudaError_t launch_typed(const FusedLaunch &L, cudaStream_t s) {
     P.slot_bytes = slot_bytes<T, TY>();
     P.inject_timeout_us = L.inject_timeout_us;
     P.first = L.first;
-    kern<<<L.grid, block_threads<TY>(), smem, s>>>(P);
-    return cudaGetLastError();
+    return launch_overlapped(kern, L.grid, block_threads<TY>(), smem, s, P, !P.step && L.overlap);
 }
 
 template <typename T, int TY>

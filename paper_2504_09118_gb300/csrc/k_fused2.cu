@@ -66,7 +66,7 @@ template <typename T> struct Geom2 {
 
 struct Fused2Params {
     const TileRec *recs;
-    const long long *step;   // batch step clock (NULL: a single cavity, no tile is skipped)
+    long long *step;         // batch step clock and a CTA count (NULL: a single cavity, no tile is skipped)
     int launch_steps;        // 2, or 1: level 1 only
     int ntiles;
     int parity;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
     const int t_step = P.first ? 1 : (int)gridDim.x;
     // Steps a tile takes in this launch: min(launch_steps, stop - clock); a batch member with one step
     // left stores its level-1 result, a finished member's tiles are skipped (producer and consumers alike).
-    const long long clock = BATCH ? *P.step : 0;
+    long long *const s_clock = reinterpret_cast<long long *>(smem + 136);
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
@@ -166,11 +166,29 @@ __global__ void __launch_bounds__(threads2<TY>(), 1) fused2_step_kernel(const Fu
         }
         fence_mbarrier_init();
         fence_proxy_async_smem();
+        if (BATCH) {
+            // the clock as the previous launch left it; the last CTA to have read it moves it past this launch (a
+            // counter launch after every batch launch cost 2-4 us of 75-150)
+            grid_wait_previous();
+            const long long c = *(volatile long long *)P.step;
+            *s_clock = c;
+            __threadfence();
+            unsigned long long *const count = reinterpret_cast<unsigned long long *>(P.step + 1);
+            if (atomicAdd(count, 1ull) == gridDim.x - 1) {
+                *(volatile unsigned long long *)count = 0;
+                *(volatile long long *)P.step = c + P.launch_steps;
+            }
+        }
     }
     __syncthreads();
+    grid_launch_dependents();
+    const long long clock = BATCH ? *s_clock : 0;
 
     // =========================================================== producer warp
     if (warp == NCW) {
+        // everything before reads launch-constant records only (a batch's clock: above); the consumers' stores follow
+        // data loaded after this
+        grid_wait_previous();
         int issued = 0, m = 0, s = 0;
         uint32_t rnd = 0;
         bool ok = true;
@@ -580,8 +598,7 @@ cudaError_t launch2_typed(const FusedLaunch &L, cudaStream_t s) {
     P.stages = L.stages;
     P.slot_bytes = slot2_bytes<T, TY, CM>();
     P.first = L.first;
-    kern<<<L.grid, threads2<TY>(), smem, s>>>(P);
-    return cudaGetLastError();
+    return launch_overlapped(kern, L.grid, threads2<TY>(), smem, s, P, L.overlap);
 }
 
 template <typename T, int TY>

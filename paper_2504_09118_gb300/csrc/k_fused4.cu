@@ -129,9 +129,12 @@ __global__ void __launch_bounds__(block_threads4<TY>(), (TY <= 4 ? 2 : 1)) fused
         fence_proxy_async_smem();
     }
     __syncthreads();
+    if (!P.step) grid_launch_dependents();   // a single cavity (a batch's launches read the clock above)
 
     // =========================================================== producer warp
     if (warp == TY + 3) {
+        // everything before reads launch-constant records only; the consumers' stores follow data loaded after this
+        if (!P.step) grid_wait_previous();
         int issued = 0, m = 0, s = 0;
         uint32_t rnd = 0;
         bool ok = true;
@@ -501,8 +504,7 @@ cudaError_t launch4_typed(const FusedLaunch &L, cudaStream_t s) {
     P.slot_bytes = slot_bytes4<T, TY>();
     P.first = L.first;
     P.inject_timeout_us = L.inject_timeout_us;
-    kern<<<L.grid, block_threads4<TY>(), smem, s>>>(P);
-    return cudaGetLastError();
+    return launch_overlapped(kern, L.grid, block_threads4<TY>(), smem, s, P, !P.step && L.overlap);
 }
 
 template <typename T, int TY>

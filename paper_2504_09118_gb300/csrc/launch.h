@@ -32,7 +32,9 @@ int reduction_blocks();
 
 struct FusedLaunch {
     const TileRec *recs;       // device array, one record per tile
-    const long long *step;     // device step clock compared with TileRec::stop (NULL: no tile skipped)
+    // device step clock compared with TileRec::stop (NULL: no tile skipped), then a CTA count: the two-step kernel
+    // (one row per warp) moves the clock itself, after the others launch_step_counter does
+    long long *step;
     int ntiles;
     int parity;
     int *status;
@@ -44,8 +46,31 @@ struct FusedLaunch {
                                // (NULL: CTA b takes tiles b, b + grid, b + 2 grid, ...)
     int launch_steps;          // two-step kernel: 2, or 1 (every tile stores its level-1 result only)
     int rows_per_warp;         // two-step kernel: 1 (k_fused2.cu) or 2 (k_fused2r.cu); 0 means 1
+    bool overlap;              // start as SMs fall free of the launch before (launch_overlapped)
     int coef_class;            // CoefClass shared by every tile (COEF_CLASS_ANY*: read from each record)
 };
+// Launch a kernel whose CTAs may start while the previous kernel of the stream ends (it calls grid_wait_previous
+// before it touches the fields).  Back to back, a tiled launch otherwise pays its launch latency, barrier set-up and
+// first ring fill after the slowest CTA of the launch before it: per launch 2-4 us of 30-40 (200 x 131 x 120 BF16: a
+// 64-step pass 1.44 -> 1.34 ms; 160 x 150 x 140 per-position 1.49 -> 1.39 ms).  CTAs started that way land on the SMs
+// in the order these fall free, which costs long launches more than it saves (512^3 FP32: 122.4 -> 124.8 ms for 100
+// launches), so launches over kOverlapCells cells start after the previous one.
+constexpr long long kOverlapCells = 30000000;
+template <typename Kernel, typename Params>
+inline cudaError_t launch_overlapped(Kernel kern, int grid, int threads, int smem, cudaStream_t s, const Params &p,
+                                     bool overlap) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
 // Coefficient layout shared by all tiles of a launch, so that a kernel can be compiled for it.
 enum CoefClass : int {
     COEF_CLASS_ANY = 0,        // tiles may differ (batches of mixed members): the record's mode decides
@@ -118,7 +143,8 @@ bool resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]);
 size_t resident_word_bytes(int nz, const int parts[3]);
 cudaError_t launch_resident(const ResidentParams &P, cudaStream_t s);
 
-// Adds inc to the device step clock of a batch (one thread; ordered after the launch it follows).
+// Adds inc to the device step clock of a batch (one thread; ordered after the launch it follows; not for the two-step
+// kernel with one row per warp).
 cudaError_t launch_step_counter(long long *counter, int inc, cudaStream_t s);
 // Two-step (temporal blocking) kernel: output tile width along x, shared memory, occupancy, launch.
 int fused2_tile_w(int storage);
