@@ -368,7 +368,8 @@ FDTD_API const char *fdtd_batch_last_error(const fdtd_batch *b);
  * refreshed from the neighbours' owned cells, the owned cells stay exact for floor(ghost / reach)
  * steps; fdtd_step returns FDTD_ERR_STATE for more.  The owned values are then bit-identical to
  * the same cells of the undivided cavity (FP32 storage; 16-bit storage as well when every slab
- * stores with the same scales, see fdtd_set_storage_scales).
+ * stores with the same scales, see fdtd_set_storage_scales, and both run the same kernel with the
+ * same steps per launch: under AUTO a small undivided cavity rounds once per call).
  * ------------------------------------------------------------------------ */
 
 /* fdtd_create_slab - the slab [k0, k1) of an nx*ny*nz_global cavity, with g_lo = (k0 > 0 ? ghost : 0)
@@ -407,8 +408,9 @@ FDTD_API int fdtd_slab_export(fdtd_ctx *ctx, int side, void *buf, int on_device)
 FDTD_API int fdtd_slab_import(fdtd_ctx *ctx, int side, const void *buf, int on_device);
 
 /* fdtd_slab_exchange - both directions between two neighbouring slabs (lo's k1 == hi's k0), device to
- * device (the same GPU, or two GPUs through unified addressing): lo's highest owned cells into hi's
- * lower ghosts and hi's lowest owned cells into lo's upper ghosts.  The copies run on lo's stream after
+ * device (the same GPU: one kernel for both directions; two GPUs: copies through unified addressing):
+ * lo's highest owned cells into hi's lower ghosts and hi's lowest owned cells into lo's upper ghosts.
+ * They run on lo's stream after
  * the work already enqueued on hi's stream, and hi's stream waits for them; no host synchronisation.
  * FDTD_ERR_ARG for slabs that are not neighbours or differ in size, storage, ghost depth or scales. */
 FDTD_API int fdtd_slab_exchange(fdtd_ctx *lo, fdtd_ctx *hi);

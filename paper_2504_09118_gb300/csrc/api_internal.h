@@ -65,6 +65,7 @@ struct fdtd_ctx {
     int nx = 0, ny = 0, nz = 0;
     double dt = 0, dx = 0;
     int storage = 0;
+    int device = 0;
     cudaStream_t stream = nullptr;
     int pitch = 0;
     size_t arr_elems = 0;

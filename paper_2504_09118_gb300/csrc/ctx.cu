@@ -472,6 +472,7 @@ int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, co
     c->dx = dx;
     c->courant = courant;
     c->storage = storage;
+    cudaGetDevice(&c->device);
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     c->pitch = (nx + 31) / 32 * 32;
     c->arr_elems = (size_t)c->pitch * ny * nz;
