@@ -35,8 +35,9 @@
 // carry them a plane; HBM-side bound like the others.  160 x 150 x 140 FP32, ce varying: 24.7 us a step
 // (60 B per cell and two steps: 4.1 TB/s, from L2 in part) against 77 us for the unfused kernels (96 B a
 // step and latency-bound).  The kernel is compiled per coefficient class (CoefClass), so a single
-// cavity's launch tests its coefficient layout nowhere; batches keep a runtime class and the general
-// body.
+// cavity's launch tests its coefficient layout nowhere.  Batches keep a runtime class: with 8 and 12 rows a
+// steady body per layout, picked per tile (48 cavities of sides 16..96 FP32: 184 us a launch with 16 rows and the
+// general body, 144 with 12 rows), with 16 rows the general body alone.
 #include <type_traits>
 
 #include "fused_common.cuh"

@@ -3,8 +3,9 @@
 //
 // The unfused step is two launches per step (Listing 1: curl H components,
 // then curl E components), each updating one copy of the fields in place; it
-// is the debugging baseline of the fused kernel and the path for coefficient
-// sets too varied for a one-byte material id (COEF_FULL).
+// is the debugging baseline of the fused kernels and the path for coefficient
+// sets too varied for a one-byte material id (COEF_FULL) with a single step, a
+// current or a probe, or when it is asked for.
 #include <algorithm>
 
 #include "df.cuh"
