@@ -824,7 +824,11 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
     if (c->d_xclock) CK(c, cudaMemsetAsync(c->d_xclock, 0, sizeof(long long), c->stream));
     if (c->d_probe_buf)
         CK(c, cudaMemsetAsync(c->d_probe_buf, 0, sizeof(float) * (size_t)c->nprobe * c->probe_cap, c->stream));
-    c->probe_start = 0;
+    if (c->probe_start != 0) {   // graphs hold it in their probe launches
+        cudaStreamSynchronize(c->stream);
+        drop_graphs(c->graphs);
+        c->probe_start = 0;
+    }
     c->cur = 0;
     c->steps = 0;
     c->has_fields = true;

@@ -149,3 +149,33 @@ def test_multi_step_kernels_resume_after_currents(kernel):
             runs.append(cav.get_fields())
     for name, a, b in zip(ci.COMPONENTS, *runs):
         assert np.array_equal(a, b), name
+
+
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("prefetched", [False, True])
+def test_traces_after_a_reload_do_not_depend_on_graphs(storage, prefetched):
+    """Probes set after some steps, a graph captured, then a load of a state with the same scales: the recording restarts
+    at step 0, and a later step records every sample where the launches without graphs do."""
+    import torch
+    from paper_2504_09118_gb300 import Cavity
+    ce, ch, f, waves = setup()
+    s = torch.cuda.Stream()
+    traces = []
+    for graph in (0, 1):
+        with Cavity(*DIMS, DT, 1.0, ce, ch, storage, s) as cav:
+            cav.tune(kernel=2, use_graph=graph)
+            cav.set_fields(f)
+            cav.step(4)
+            cav.set_probes(PROBES, 40)
+            cav.step(16)
+            before = cav.get_probes()
+            if prefetched:
+                cav.prefetch_fields(f)
+                cav.set_fields_prefetched()
+            else:
+                cav.set_fields(f)
+            cav.step(16)
+            traces.append((before, cav.get_probes()))
+            assert traces[-1][0].shape == traces[-1][1].shape == (len(PROBES), 16)
+    for a, b in zip(*traces):
+        np.testing.assert_array_equal(a, b)
