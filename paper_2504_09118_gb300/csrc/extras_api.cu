@@ -59,10 +59,10 @@ static int free_extras(fdtd_ctx *c, bool sources, bool probes) {
     return FDTD_OK;
 }
 
-// The device step clock, started at the context's step count when the first current or probe is set.
-static int ensure_xclock(fdtd_ctx *c) {
-    if (c->d_xclock) return FDTD_OK;
-    CK(c, pool_alloc((void **)&c->d_xclock, sizeof(long long), c->stream));
+// The device step clock, set to the context's step count whenever currents or probes are set: steps taken without
+// either do not move it.
+static int set_xclock(fdtd_ctx *c) {
+    if (!c->d_xclock) CK(c, pool_alloc((void **)&c->d_xclock, sizeof(long long), c->stream));
     const long long n = c->steps;
     CK(c, cudaMemcpyAsync(c->d_xclock, &n, sizeof n, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
@@ -99,7 +99,7 @@ int fdtd_set_sources(fdtd_ctx *c, int nsrc, const int *comp, const int *ijk, con
     CK(c, cudaStreamSynchronize(c->stream));
     c->nsrc = nsrc;
     c->wave_len = wave_len;
-    return ensure_xclock(c);
+    return set_xclock(c);
 }
 
 int fdtd_set_probes(fdtd_ctx *c, int nprobe, const int *comp, const int *ijk, int capacity) {
@@ -125,7 +125,7 @@ int fdtd_set_probes(fdtd_ctx *c, int nprobe, const int *comp, const int *ijk, in
     c->nprobe = nprobe;
     c->probe_cap = capacity;
     c->probe_start = c->steps;
-    return ensure_xclock(c);
+    return set_xclock(c);
 }
 
 int fdtd_get_probes(fdtd_ctx *c, float *out, int *nrecorded) {

@@ -179,3 +179,26 @@ def test_traces_after_a_reload_do_not_depend_on_graphs(storage, prefetched):
             assert traces[-1][0].shape == traces[-1][1].shape == (len(PROBES), 16)
     for a, b in zip(*traces):
         np.testing.assert_array_equal(a, b)
+
+
+def test_probes_set_again_after_steps_without_any():
+    """Steps taken while no current or probe is set count for the next recording too."""
+    from paper_2504_09118_gb300 import Cavity
+    ce, ch, f, waves = setup()
+    traces = []
+    for again in (False, True):
+        with Cavity(*DIMS, DT, 1.0, ce, ch) as cav:
+            cav.tune(kernel=2)
+            cav.set_fields(f)
+            if again:
+                cav.set_probes(PROBES[:1], 5)
+                cav.step(3)
+                cav.set_probes([], 1)
+                cav.step(7)
+            else:
+                cav.step(10)
+            cav.set_probes(PROBES, 12)
+            cav.step(9)
+            traces.append(cav.get_probes())
+            assert traces[-1].shape == (len(PROBES), 9)
+    np.testing.assert_array_equal(*traces)
