@@ -256,7 +256,11 @@ int read_reductions(fdtd_ctx *c, const CavityDesc &d, int what, double out[3]) {
 // above kDirectStoreBytes an output may be fresh memory, whose pages a kernel's first touch maps much more slowly
 // than a copy does (1.6 MB: 5.6 against 1.9 ms).
 constexpr size_t kDirectLoadBytes = 16 << 20, kDirectStoreBytes = 1 << 20;
-static bool gpu_reads_host() {
+// Arrays that do not start at a multiple of 4 bytes (a view into a packed buffer) are left to the copies, which take
+// any address.
+template <typename T> static bool gpu_reads_host(T *const f[6]) {
+    for (int q = 0; q < 6; ++q)
+        if (reinterpret_cast<uintptr_t>(f[q]) % sizeof(float)) return false;
     int dev = 0, v = 0;
     return cudaGetDevice(&dev) == cudaSuccess &&
            cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) == cudaSuccess && v != 0;
@@ -735,7 +739,7 @@ int fdtd_set_fields(fdtd_ctx *c, const float *const f[6], int on_device) {
     if (c->batch) return fail(c, FDTD_ERR_STATE, "context is a batch member; remove it first");
     const size_t n = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
     // whether the kernels read f itself: device arrays, or small host arrays
-    const bool direct = on_device || (6 * n * 4 <= kDirectLoadBytes && gpu_reads_host());
+    const bool direct = on_device || (6 * n * 4 <= kDirectLoadBytes && gpu_reads_host(f));
     if (!direct)
         if (int rc = ensure_stage(c)) return rc;
     // scales for 16-bit storage: s_c = 2^(8 - ceil(log2 max|F_c|))
@@ -882,7 +886,7 @@ int fdtd_get_fields(fdtd_ctx *c, float *const f[6], int on_device) {
         if (!f[q]) return fail(c, FDTD_ERR_ARG, "field %d is NULL", q);
     if (c->batch) return fail(c, FDTD_ERR_STATE, "context is a batch member; remove it first");
     const size_t n = (size_t)(c->nx + 1) * (c->ny + 1) * (c->nz + 1);
-    const bool direct = on_device || (6 * n * 4 <= kDirectStoreBytes && gpu_reads_host());
+    const bool direct = on_device || (6 * n * 4 <= kDirectStoreBytes && gpu_reads_host(f));
     if (!direct)
         if (int rc = ensure_stage(c)) return rc;
     CavityDesc d = make_desc(c, 0);

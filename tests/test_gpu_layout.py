@@ -116,3 +116,32 @@ def test_reloads_with_equal_and_other_scales_match_a_fresh_context(tuning, stora
                 want = solve(fresh, e, h, sources)
             for a, b in zip(got, want):
                 np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+def test_host_arrays_at_any_address(offset, storage):
+    """Views into packed buffers, contiguous but not at a multiple of 4 bytes: one such array among six, and all six, load
+    and read back like aligned ones."""
+    from paper_2504_09118_gb300 import Cavity
+    dims = (9, 8, 7)
+    shape = tuple(n + 1 for n in reversed(dims))
+    full, _ = _state(dims, 5)
+
+    def view(a=None):
+        raw = np.zeros(4 * int(np.prod(shape)) + 8, np.uint8)
+        v = np.frombuffer(raw.data, np.float32, int(np.prod(shape)), offset + (-raw.ctypes.data) % 4).reshape(shape)
+        assert v.ctypes.data % 4 == offset and v.flags.c_contiguous and v.flags.writeable
+        if a is not None:
+            v[:] = a
+        return v
+
+    with Cavity(*dims, ci.COURANT_HALF_DT, storage=storage) as cav:
+        cav.set_fields(full)
+        want = cav.get_fields()
+        for which in (range(6), [4]):
+            cav.set_fields([view(a) if c in which else a for c, a in enumerate(full)])
+            out = [view() if c in which else np.empty(shape, np.float32) for c in range(6)]
+            cav.get_fields(out)
+            for a, b in zip(out, want):
+                np.testing.assert_array_equal(a, b)
