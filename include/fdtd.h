@@ -408,7 +408,7 @@ FDTD_API int fdtd_slab_export(fdtd_ctx *ctx, int side, void *buf, int on_device)
 FDTD_API int fdtd_slab_import(fdtd_ctx *ctx, int side, const void *buf, int on_device);
 
 /* fdtd_slab_exchange - both directions between two neighbouring slabs (lo's k1 == hi's k0), device to
- * device (the same GPU: one kernel for both directions; two GPUs: copies through unified addressing):
+ * device (both on the current device: one kernel for both directions; else copies through unified addressing):
  * lo's highest owned cells into hi's lower ghosts and hi's lowest owned cells into lo's upper ghosts.
  * They run on lo's stream after
  * the work already enqueued on hi's stream, and hi's stream waits for them; no host synchronisation.
@@ -485,6 +485,11 @@ FDTD_API int fdtd_debug_tile_plan(long long cols, int nz, int ctas, int prologue
  * Both return FDTD_ERR_ARG for NULL pointers or arguments outside those ranges. */
 FDTD_API int fdtd_debug_pec_code(int ntab, int id, int i, int j, int k, int *code);
 FDTD_API int fdtd_debug_pec_table(const float *tab, int ntab, float *out);
+
+/* fdtd_debug_exchange_route - host only: how fdtd_slab_exchange carries out an exchange between slabs created on these
+ * devices with current_device current: bit 0 set for the kernel (else copies), bit 1 for events that order the slabs'
+ * streams (same_stream: both slabs were given the same stream handle). */
+FDTD_API int fdtd_debug_exchange_route(int lo_device, int hi_device, int current_device, int same_stream);
 
 /*
  * fdtd_energy_static - the same energy W as fdtd_energy (second-order scheme), computed from

@@ -34,7 +34,7 @@ EXPORTS = (
     "fdtd_batch_steps_done", "fdtd_autotune", "fdtd_batch_autotune", "fdtd_set_sources", "fdtd_set_probes",
     "fdtd_get_probes", "fdtd_set_order", "fdtd_get_order", "fdtd_batch_retune", "fdtd_prefetch_fields",
     "fdtd_set_fields_prefetched", "fdtd_debug_fail_alloc", "fdtd_debug_tile_plan", "fdtd_debug_pec_code",
-    "fdtd_debug_pec_table",
+    "fdtd_debug_pec_table", "fdtd_debug_exchange_route",
     "fdtd_create_slab", "fdtd_slab_info", "fdtd_slab_halo_bytes", "fdtd_slab_export", "fdtd_slab_import",
     "fdtd_slab_exchange", "fdtd_slab_energy", "fdtd_slab_divergence_sq", "fdtd_set_storage_scales",
     "fdtd_storage_scale_of",
@@ -117,6 +117,7 @@ def lib() -> ctypes.CDLL:
             L.fdtd_debug_tile_plan.argtypes = [ll, i, i, i, i, vp, i, ctypes.POINTER(i), ctypes.POINTER(ll), vp]
             L.fdtd_debug_pec_code.argtypes = [i, i, i, i, i, ctypes.POINTER(i)]
             L.fdtd_debug_pec_table.argtypes = [vp, i, vp]
+            L.fdtd_debug_exchange_route.argtypes = [i, i, i, i]
             L.fdtd_set_fields_prefetched.argtypes = [vp]
             L.fdtd_batch_retune.argtypes = [vp, i, ctypes.POINTER(fdtd_tuning), ctypes.POINTER(d),
                                             ctypes.POINTER(i)]
@@ -365,6 +366,12 @@ def fdtd_debug_pec_table(tab) -> np.ndarray:
     if rc != FDTD_OK:
         raise FdtdError(rc, "fdtd_debug_pec_table: invalid arguments")
     return out
+
+
+def fdtd_debug_exchange_route(lo_device: int, hi_device: int, current_device: int, same_stream: bool) -> tuple[bool, bool]:
+    """Host-only: whether fdtd_slab_exchange runs its kernel (else copies) and whether it orders the streams by events."""
+    r = int(lib().fdtd_debug_exchange_route(int(lo_device), int(hi_device), int(current_device), int(bool(same_stream))))
+    return bool(r & 1), bool(r & 2)
 
 
 def fdtd_set_fields_prefetched(ctx) -> None:

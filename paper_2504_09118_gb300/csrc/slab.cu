@@ -94,6 +94,15 @@ __global__ void __launch_bounds__(kExThreads) exchange_kernel(const ExchangePara
         if (i0 + u * kExThreads < P.n) d[i0 + u * kExThreads] = v[u];
 }
 
+// How an exchange is carried out: by the kernel when both slabs live on the current device (a launch goes to the current
+// device and its default stream), else by copies, which unified addressing takes from any device.  The slabs' streams
+// need no events when they are one stream of that device.
+enum ExchangeRoute { EXCHANGE_KERNEL = 1, EXCHANGE_EVENTS = 2 };
+int exchange_route(int lo_device, int hi_device, int current_device, bool same_stream) {
+    const bool here = lo_device == hi_device && lo_device == current_device;
+    return (here ? EXCHANGE_KERNEL : 0) | (here && same_stream ? 0 : EXCHANGE_EVENTS);
+}
+
 bool current(const fdtd_ctx *c) {
     const int full = slab_budget(c);
     return (c->slab.g_lo == 0 || c->slab.left[0] == full) && (c->slab.g_hi == 0 || c->slab.left[1] == full);
@@ -181,6 +190,10 @@ int fdtd_slab_import(fdtd_ctx *c, int side, const void *buf, int on_device) {
     return FDTD_OK;
 }
 
+int fdtd_debug_exchange_route(int lo_device, int hi_device, int current_device, int same_stream) {
+    return exchange_route(lo_device, hi_device, current_device, same_stream != 0);
+}
+
 int fdtd_slab_exchange(fdtd_ctx *lo, fdtd_ctx *hi) {
     NvtxRange nvtx_range("fdtd_slab_exchange");
     if (!lo || !hi || lo == hi) return fail(lo, FDTD_ERR_ARG, "two distinct slab contexts are needed");
@@ -194,8 +207,10 @@ int fdtd_slab_exchange(fdtd_ctx *lo, fdtd_ctx *hi) {
     if (lo->scale[0] != hi->scale[0] || lo->scale[3] != hi->scale[3])
         return fail(lo, FDTD_ERR_ARG, "16-bit slabs need equal storage scales (fdtd_set_storage_scales)");
     // both directions run on lo's stream after hi's earlier work; hi's later work waits for them
-    const bool one_stream = lo->stream == hi->stream && lo->device == hi->device;
-    if (!one_stream) {
+    int device = -1;
+    CK(lo, cudaGetDevice(&device));
+    const int route = exchange_route(lo->device, hi->device, device, lo->stream == hi->stream);
+    if (route & EXCHANGE_EVENTS) {
         CK(lo, cudaEventRecord(hi->slab.ev, hi->stream));
         CK(lo, cudaStreamWaitEvent(lo->stream, hi->slab.ev, 0));
     }
@@ -206,7 +221,7 @@ int fdtd_slab_exchange(fdtd_ctx *lo, fdtd_ctx *hi) {
     char *lo_ghost = static_cast<char *>(lo->fields[lo->cur][0]) + (size_t)import_plane(lo, 1) * pb;
     const char *hi_own = static_cast<const char *>(hi->fields[hi->cur][0]) + (size_t)export_plane(hi, 0) * pb;
     char *hi_ghost = static_cast<char *>(hi->fields[hi->cur][0]) + (size_t)import_plane(hi, 0) * pb;
-    if (lo->device == hi->device && width / 16 < (size_t)UINT_MAX) {
+    if ((route & EXCHANGE_KERNEL) && width / 16 < (size_t)UINT_MAX) {
         ExchangeParams P{};
         P.src[0] = reinterpret_cast<const uint4 *>(lo_own);
         P.dst[0] = reinterpret_cast<uint4 *>(hi_ghost);
@@ -229,7 +244,7 @@ int fdtd_slab_exchange(fdtd_ctx *lo, fdtd_ctx *hi) {
         CK(lo, cudaMemcpy2DAsync(hi_ghost, sp_hi, lo_own, sp_lo, width, 6, cudaMemcpyDefault, lo->stream));
         CK(lo, cudaMemcpy2DAsync(lo_ghost, sp_lo, hi_own, sp_hi, width, 6, cudaMemcpyDefault, lo->stream));
     }
-    if (!one_stream) {
+    if (route & EXCHANGE_EVENTS) {
         CK(lo, cudaEventRecord(lo->slab.ev, lo->stream));
         CK(lo, cudaStreamWaitEvent(hi->stream, lo->slab.ev, 0));
     }
