@@ -436,7 +436,7 @@ template <typename T, int TY>
 cudaError_t launch_typed(const FusedLaunch &L, cudaStream_t s) {
     const int smem = smem_bytes<T, TY>(L.stages);
     auto kern = fused_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     FusedParams P;
     P.recs = L.recs;
@@ -455,7 +455,7 @@ template <typename T, int TY>
 cudaError_t occupancy_typed(int stages, int *n) {
     const int smem = smem_bytes<T, TY>(stages);
     auto kern = fused_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, block_threads<TY>(), smem);
 }

@@ -587,7 +587,7 @@ template <typename T, int TY, bool BATCH, int CM>
 cudaError_t launch2_typed(const FusedLaunch &L, cudaStream_t s) {
     const int smem = smem2_bytes<T, TY, CM>(L.stages);
     auto kern = fused2_step_kernel<T, TY, BATCH, CM>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     Fused2Params P;
     P.recs = L.recs;
@@ -606,7 +606,7 @@ template <typename T, int TY>
 cudaError_t occupancy2_typed(int stages, int *n) {
     const int smem = smem2_bytes<T, TY>(stages);
     auto kern = fused2_step_kernel<T, TY, false, COEF_CLASS_ID_UNIFORM_H>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, threads2<TY>(), smem);
 }

@@ -498,7 +498,7 @@ template <typename T, int TY, bool BATCH>
 cudaError_t launchr_typed(const FusedLaunch &L, cudaStream_t s) {
     const int smem = smemr_bytes<T, TY>(L.stages);
     auto kern = fused2r_step_kernel<T, TY, BATCH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     FusedRParams P;
     P.recs = L.recs;
@@ -518,7 +518,7 @@ template <typename T, int TY>
 cudaError_t occupancyr_typed(int stages, int *n) {
     const int smem = smemr_bytes<T, TY>(stages);
     auto kern = fused2r_step_kernel<T, TY, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, threadsr<TY>(), smem);
 }

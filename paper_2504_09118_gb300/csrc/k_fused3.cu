@@ -424,7 +424,7 @@ template <typename T, int TY>
 cudaError_t launch3_typed(const FusedLaunch &L, cudaStream_t s) {
     const int smem = smem3_bytes<T, TY>(L.stages);
     auto kern = fused3_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     Fused3Params P;
     P.recs = L.recs;
@@ -442,7 +442,7 @@ template <typename T, int TY>
 cudaError_t occupancy3_typed(int stages, int *n) {
     const int smem = smem3_bytes<T, TY>(stages);
     auto kern = fused3_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, threads3<TY>(), smem);
 }

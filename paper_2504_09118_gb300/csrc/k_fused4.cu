@@ -492,7 +492,7 @@ template <typename T, int TY>
 cudaError_t launch4_typed(const FusedLaunch &L, cudaStream_t s) {
     const int smem = smem_bytes4<T, TY>(L.stages);
     auto kern = fused4_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     Fused4Params P;
     P.recs = L.recs;
@@ -511,7 +511,7 @@ template <typename T, int TY>
 cudaError_t occupancy4_typed(int stages, int *n) {
     const int smem = smem_bytes4<T, TY>(stages);
     auto kern = fused4_step_kernel<T, TY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kern, block_threads4<TY>(), smem);
 }

@@ -558,7 +558,7 @@ template <int BZ, bool HID> cudaError_t launch_typed(const ResidentParams &P, in
     if (!p.id) p.ntab = 9;
     const int smem = smem_bytes<BZ>(p.ntab, p.X.nsrc, p.X.nprobe);
     auto kern = resident_kernel<BZ, HID>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_all_smem(kern, 64);   // static: 32 bytes
     if (e != cudaSuccess) return e;
     void *args[] = {&p};
     return cudaLaunchCooperativeKernel((const void *)kern, dim3(ctas), dim3(NT), args, smem, s);

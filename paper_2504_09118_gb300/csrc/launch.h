@@ -49,6 +49,14 @@ struct FusedLaunch {
     bool overlap;              // start as SMs fall free of the launch before (launch_overlapped)
     int coef_class;            // CoefClass shared by every tile (COEF_CLASS_ANY*: read from each record)
 };
+// Lets launches of a kernel instance use all the dynamic shared memory a block can have (227 KB less the instance's own
+// static part).  The limit belongs to the function, not to a launch: the same value every time, so that host threads
+// launching one instance with different needs (ring depths, material tables, probes) never lower it for each other.
+constexpr int kMaxSmem = 227 * 1024;
+template <typename Kernel> inline cudaError_t allow_all_smem(Kernel kern, int static_bytes = 0) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem - static_bytes);
+}
+
 // Launch a kernel whose CTAs may start while the previous kernel of the stream ends (it calls grid_wait_previous
 // before it touches the fields).  Back to back, a tiled launch otherwise pays its launch latency, barrier set-up and
 // first ring fill after the slowest CTA of the launch before it: per launch 2-4 us of 30-40 (200 x 131 x 120 BF16: a

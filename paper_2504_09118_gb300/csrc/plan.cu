@@ -16,7 +16,7 @@ Shape resolve_shape(int storage, const fdtd_tuning &t, int kind, bool full_ch) {
         s.tile_y = kFullTileY;
         const int cls = full_ch ? COEF_CLASS_FULL : COEF_CLASS_FULL_UNIFORM_H;
         s.stages = (t.stages >= 3 && t.stages <= 8) ? t.stages : 6;
-        while (s.stages > 3 && fused2_full_smem_bytes(storage, cls, s.stages) > 227 * 1024) --s.stages;
+        while (s.stages > 3 && fused2_full_smem_bytes(storage, cls, s.stages) > kMaxSmem) --s.stages;
         s.ctas_per_sm = 1;
         return s;
     }
@@ -41,7 +41,7 @@ Shape resolve_shape(int storage, const fdtd_tuning &t, int kind, bool full_ch) {
                : kind == 3 ? fused3_smem_bytes(storage, s.tile_y, st)
                            : fused4_smem_bytes(storage, s.tile_y, st);
     };
-    while (s.stages > min_st && smem(s.stages) > 227 * 1024) --s.stages;
+    while (s.stages > min_st && smem(s.stages) > kMaxSmem) --s.stages;
     const int key = (((kind * 4 + storage) * 64 + s.tile_y) * 16 + s.stages) * 4 + s.rows_per_warp;
     int occ = 0;
     {
