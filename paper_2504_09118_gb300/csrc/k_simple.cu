@@ -323,7 +323,7 @@ template <typename T> __device__ __forceinline__ float2 ld_pair(const CavityDesc
 // values, scaled once.
 // Bound by the compensated FP32 arithmetic and the latency of the loads that 24 warps per SM (80 registers) leave:
 // packed pairs and separate accumulator chains against one cell and one chain per lane took the energy of 320^3
-// FP32 cells from 369 to 300 us and the divergences from 645 to 386 us (a DRAM pass over the state is 121 us).
+// FP32 cells from 369 to 300 us and the divergences from 645 to 389 us (a DRAM pass over the state is 121 us).
 // Two blocks per SM (99-120 registers) 306 and 500 us; an L2 prefetch of the warp's next row: no gain.
 template <typename T, int WHAT, bool CHC>
 __global__ void __launch_bounds__(kRedThreads, kRedPerSM) reduce_kernel(const CavityDesc d, int copy, double *partial) {
@@ -343,6 +343,8 @@ __global__ void __launch_bounds__(kRedThreads, kRedPerSM) reduce_kernel(const Ca
     }
     const df::F2 ich = df::recip(d.ch[0]);   // CHC
     const df::F22 ich2{make_float2(ich.hi, ich.hi), make_float2(ich.lo, ich.lo)};
+    const float pch = exp2f((float)ilogbf(ich.hi));   // the power of two at or below 1/ch
+    const float2 pch2 = make_float2(pch, pch);
     __syncthreads();
     const float2 zero = make_float2(0.f, 0.f);
     // material ids of the two cells at off (packed), and 1/ce or 1/ch (c) of them
@@ -437,13 +439,19 @@ __global__ void __launch_bounds__(kRedThreads, kRedPerSM) reduce_kernel(const Ca
                 hy1 = j + 1 < ny ? F(4, o + P) : face2(d.face[1], fy);
                 hz1 = k + 1 < nz ? F(5, o + Z) : face2(d.face[2], fz);
                 if (CHC) {   // the difference as an exact sum; 1/ch^2 scales the total
+                    // The leading part u cancels where the field is free of divergence, and what the sum's roundings
+                    // left can exceed it: the pair is normalised before it is squared.  Then times the power of two
+                    // next to 1/ch, so that weak fields square within the same range as H / ch does.
                     float2 x, exx, y, eyy, z, ezz, t, et, u, eu;
                     df::two_diff2(hx1, hx, x, exx);
                     df::two_diff2(hy1, hy, y, eyy);
                     df::two_diff2(hz1, hz, z, ezz);
                     df::two_sum2(x, y, t, et);
                     df::two_sum2(t, z, u, eu);
-                    df::F22 v{u, df::add2(df::add2(df::add2(exx, eyy), df::add2(ezz, et)), eu)};
+                    df::F22 v;
+                    df::two_sum2(u, df::add2(df::add2(df::add2(exx, eyy), df::add2(ezz, et)), eu), v.hi, v.lo);
+                    v.hi = df::mul2(v.hi, pch2);
+                    v.lo = df::mul2(v.lo, pch2);
                     if (!two) v.hi.y = v.lo.y = 0.f;
                     a1.square(v);
                 } else {
@@ -502,7 +510,7 @@ __global__ void __launch_bounds__(kRedThreads, kRedPerSM) reduce_kernel(const Ca
             s0 += h * h * (CHC ? 1.0 / (double)d.ch[0] : face_inv_ch64(d, c, fi));
         }
     } else if (CHC) {
-        const double q = 1.0 / (double)d.ch[0];
+        const double q = 1.0 / ((double)d.ch[0] * (double)pch);
         s1 *= q * q;
     }
     const double a = block_sum(s0, sh);

@@ -56,3 +56,25 @@ def test_equal_the_fp64_sums_of_the_stored_state(dims, kind, storage):
     # terms to about 2^-48 each, summed without cancellation beyond the state's own size
     scale = np.maximum(np.abs(ref), 1e-3 * np.abs(ref).max())
     assert np.all(np.abs(got - ref) <= 1e-12 * scale), (got, ref)
+
+
+@pytest.mark.parametrize("storage,scale", [(0, 1.0), (0, 2.0 ** -36), (1, 1.0)])
+@pytest.mark.parametrize("dims", [(33, 12, 9), (64, 5, 4)])
+def test_divergence_of_a_divergence_free_field(dims, storage, scale):
+    """H = curl E of a few steps from H = 0, in SI units (ch about 1e-3), also of a weak field: the six values of a cell
+    cancel but for their own roundings, which is what the divergence measures.  A cell's sum is exact to a few 2^-48 of
+    its terms, and so is the norm over the cells."""
+    from paper_2504_09118_gb300 import Cavity
+    dx, dt = 1e-3, 1.9e-12
+    full = [np.full(tuple(n + 1 for n in reversed(dims)), v, np.float32)
+            for v in (dt / (8.8541878128e-12 * dx), dt / (1.25663706212e-6 * dx))]
+    f = [a * np.float32(scale if c < 3 else 0.0) for c, a in enumerate(ci.random_fields(43, *dims))]
+    with Cavity(*dims, dt, dx, full[:1] * 3, full[1:] * 3, storage) as cav:
+        cav.set_fields(f)
+        cav.step(3)
+        got = cav.divergence()[1]
+        stored = oracle.as_f64(cav.get_fields())
+    c64 = [[v.astype(np.float64)] * 3 for v in full]
+    ref = np.linalg.norm(oracle.divergence(stored, *c64)[1])
+    terms = sum(float(np.linalg.norm(a)) for a in stored[3:]) / float(full[1].flat[0])
+    assert ref > 0 and abs(got - ref) <= 8 * 2.0 ** -48 * terms, (got, ref)
