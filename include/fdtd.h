@@ -491,6 +491,10 @@ FDTD_API int fdtd_debug_pec_table(const float *tab, int ntab, float *out);
  * streams (same_stream: both slabs were given the same stream handle). */
 FDTD_API int fdtd_debug_exchange_route(int lo_device, int hi_device, int current_device, int same_stream);
 
+/* fdtd_debug_resident_split - host only: parts[3] receives the boxes along x, y and z that the on-chip kernel cuts a
+ * cavity into with max_ctas CTAs at most (0, 0, 0: the cavity does not fit). */
+FDTD_API int fdtd_debug_resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]);
+
 /*
  * fdtd_energy_static - the same energy W as fdtd_energy (second-order scheme), computed from
  * caller-owned device arrays by a path that allocates no device memory.  (The paper has no

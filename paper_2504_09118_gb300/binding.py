@@ -34,7 +34,7 @@ EXPORTS = (
     "fdtd_batch_steps_done", "fdtd_autotune", "fdtd_batch_autotune", "fdtd_set_sources", "fdtd_set_probes",
     "fdtd_get_probes", "fdtd_set_order", "fdtd_get_order", "fdtd_batch_retune", "fdtd_prefetch_fields",
     "fdtd_set_fields_prefetched", "fdtd_debug_fail_alloc", "fdtd_debug_tile_plan", "fdtd_debug_pec_code",
-    "fdtd_debug_pec_table", "fdtd_debug_exchange_route",
+    "fdtd_debug_pec_table", "fdtd_debug_exchange_route", "fdtd_debug_resident_split",
     "fdtd_create_slab", "fdtd_slab_info", "fdtd_slab_halo_bytes", "fdtd_slab_export", "fdtd_slab_import",
     "fdtd_slab_exchange", "fdtd_slab_energy", "fdtd_slab_divergence_sq", "fdtd_set_storage_scales",
     "fdtd_storage_scale_of",
@@ -118,6 +118,7 @@ def lib() -> ctypes.CDLL:
             L.fdtd_debug_pec_code.argtypes = [i, i, i, i, i, ctypes.POINTER(i)]
             L.fdtd_debug_pec_table.argtypes = [vp, i, vp]
             L.fdtd_debug_exchange_route.argtypes = [i, i, i, i]
+            L.fdtd_debug_resident_split.argtypes = [i, i, i, i, vp]
             L.fdtd_set_fields_prefetched.argtypes = [vp]
             L.fdtd_batch_retune.argtypes = [vp, i, ctypes.POINTER(fdtd_tuning), ctypes.POINTER(d),
                                             ctypes.POINTER(i)]
@@ -372,6 +373,15 @@ def fdtd_debug_exchange_route(lo_device: int, hi_device: int, current_device: in
     """Host-only: whether fdtd_slab_exchange runs its kernel (else copies) and whether it orders the streams by events."""
     r = int(lib().fdtd_debug_exchange_route(int(lo_device), int(hi_device), int(current_device), int(bool(same_stream))))
     return bool(r & 1), bool(r & 2)
+
+
+def fdtd_debug_resident_split(nx: int, ny: int, nz: int, max_ctas: int) -> tuple[int, int, int] | None:
+    """Host-only: boxes along x, y, z of the on-chip kernel with at most max_ctas CTAs (None: the cavity does not fit)."""
+    parts = (ctypes.c_int * 3)()
+    rc = lib().fdtd_debug_resident_split(int(nx), int(ny), int(nz), int(max_ctas), parts)
+    if rc != FDTD_OK:
+        raise FdtdError(rc, "fdtd_debug_resident_split: invalid arguments")
+    return tuple(parts) if parts[0] else None
 
 
 def fdtd_set_fields_prefetched(ctx) -> None:

@@ -359,6 +359,13 @@ int fdtd_debug_pec_table(const float *tab, int ntab, float *out) {
     return FDTD_OK;
 }
 
+int fdtd_debug_resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]) {
+    if (!parts || nx < 1 || ny < 1 || nz < 1 || max_ctas < 1) return FDTD_ERR_ARG;
+    parts[0] = parts[1] = parts[2] = 0;
+    resident_split(nx, ny, nz, max_ctas, parts);
+    return FDTD_OK;
+}
+
 const char *fdtd_last_error(const fdtd_ctx *ctx) { return ctx ? ctx->err.c_str() : g_create_error.c_str(); }
 
 int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, const float *const ce[3],

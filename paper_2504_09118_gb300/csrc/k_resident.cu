@@ -573,30 +573,23 @@ int instance_bz(int bz) { return bz <= 2 ? 2 : bz <= 4 ? 4 : bz <= 6 ? 6 : bz <=
 
 }  // namespace
 
-// The split with the shortest estimated step of the fullest CTA, then the smallest surface.  A warp works through
-// its planes one after the other (kPlaneLatency cycles each with nothing else to issue) and each of the four
-// schedulers issues its rows' instructions (kRowIssue cycles a row and plane), so of boxes with equally many
-// rows x planes the one with more rows and fewer planes wins.  Parts are equal to one cell, so the fullest CTA
-// has ceil(n / parts) per axis; lanes of a row run together whatever bx is.
-constexpr int kPlaneLatency = 60, kRowIssue = 24;
+// The split into boxes: the fewest rows and columns of boxes, then the least depth that max_ctas boxes allow, then the
+// fewest boxes of the instance for that depth.  A warp works through its planes one after the other and all warps run
+// the plane loops, so a step takes as long as the instance is deep (us a step with 2, 4, 6, 8, 11, 14 planes: 1.9, 2.4,
+// 2.8, 3.4, 4.2, 4.7) and hardly depends on the rows or columns of a box.  Boxes beyond that only keep other streams'
+// launches from the SMs: 24 x 20 x 17 cells take 1.75 us a step in 90 boxes and 1.89 in 18; eight such contexts on
+// eight streams 1.74 and 0.25 us per step and context, since several of the launches then fit at once (32^3: 128
+// boxes 1.73 and 1.71, 32 boxes 1.88 and 0.47; 18 x 11 x 22: 121 boxes 1.79 and 1.73, 11 boxes 1.54 and 0.24).
+// Parts are equal to one cell, so the fullest CTA has ceil(n / parts) per axis.
 bool resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]) {
-    long long best = -1;
-    for (int px = (nx + BXR - 1) / BXR; px <= std::min(nx, max_ctas); ++px)
-        for (int py = (ny + NW - 1) / NW; py <= std::min(ny, max_ctas / px); ++py) {
-            const int most = std::min(nz, max_ctas / (px * py));
-            const int bx = (nx + px - 1) / px, by = (ny + py - 1) / py, bz = (nz + most - 1) / most;
-            if (bz > kResidentMaxBZ) continue;
-            const int pz = (nz + bz - 1) / bz;   // no more parts than this depth needs
-            const long long cost = (long long)instance_bz(bz) * (4 * kPlaneLatency + kRowIssue * by) * 65536 +
-                                   (bx + 2) * (by + 2) * (bz + 2) - bx * by * bz;
-            if (best < 0 || cost < best) {
-                best = cost;
-                parts[0] = px;
-                parts[1] = py;
-                parts[2] = pz;
-            }
-        }
-    return best >= 0;
+    const int px = (nx + BXR - 1) / BXR, py = (ny + NW - 1) / NW;
+    if ((long long)px * py > max_ctas) return false;
+    const int most = std::min(nz, max_ctas / (px * py)), bz = (nz + most - 1) / most;
+    if (bz > kResidentMaxBZ) return false;
+    parts[0] = px;
+    parts[1] = py;
+    parts[2] = (nz + instance_bz(bz) - 1) / instance_bz(bz);
+    return true;
 }
 
 size_t resident_word_bytes(int nz, const int parts[3]) {

@@ -1,5 +1,8 @@
 """Rules that choose between launches, on the CPU through the library's host-only entry points."""
 import itertools
+import random
+
+import pytest
 
 from paper_2504_09118_gb300 import binding as B
 
@@ -11,3 +14,47 @@ def test_exchange_kernel_only_on_the_current_device():
         kernel, events = B.fdtd_debug_exchange_route(lo, hi, cur, same)
         assert kernel == (lo == hi == cur)
         assert events == (not kernel or not same)
+
+
+SMS = 152
+DEPTHS = (2, 4, 6, 8, 11, 14)   # planes of the on-chip kernel's instances
+
+
+def depth(nz, pz):
+    return next((d for d in DEPTHS if d >= -(-nz // pz)), None)
+
+
+def splits(dims, most):
+    """Every split into boxes of at most 32 x 16 x 14 cells, as (instance depth, boxes)."""
+    nx, ny, nz = dims
+    for px in range(-(-nx // 32), min(nx, most) + 1):
+        for py in range(-(-ny // 16), min(ny, most // px) + 1):
+            for pz in range(1, min(nz, most // (px * py)) + 1):
+                if depth(nz, pz):
+                    yield depth(nz, pz), px * py * pz
+
+
+def sizes():
+    rng = random.Random(4)
+    fixed = [(1, 1, 1), (16, 16, 16), (24, 20, 17), (32, 32, 32), (131, 67, 45), (128, 96, 80), (7, 150, 130), (300, 40, 9),
+             (129, 97, 90), (1, 2433, 1), (1, 2432, 14)]
+    return fixed + [tuple(int(10 ** rng.uniform(0, 2.2)) for _ in range(3)) for _ in range(24)]
+
+
+@pytest.mark.parametrize("dims", sizes())
+def test_resident_split_takes_the_least_depth_then_the_fewest_boxes(dims):
+    parts = B.fdtd_debug_resident_split(*dims, SMS)
+    every = list(splits(dims, SMS))
+    if not every:
+        assert parts is None
+        return
+    px, py, pz = parts
+    assert -(-dims[0] // px) <= 32 and -(-dims[1] // py) <= 16
+    assert (depth(dims[2], pz), px * py * pz) == min(every)
+
+
+def test_small_cavities_leave_room_for_other_launches():
+    """Eight contexts of up to 24 x 20 x 17 cells, or four of 32^3, fit on the SMs at once."""
+    for dims, most in (((16, 16, 16), SMS // 8), ((24, 20, 17), SMS // 8), ((32, 32, 32), SMS // 4)):
+        px, py, pz = B.fdtd_debug_resident_split(*dims, SMS)
+        assert px * py * pz <= most
