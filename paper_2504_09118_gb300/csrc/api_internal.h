@@ -239,6 +239,7 @@ int ensure_stage2(fdtd_ctx *c);
 // Rows per consumer warp of the two-step kernel a tuning selects.
 inline int two_step_rows(const fdtd_tuning &t) { return t.kernel == FDTD_KERNEL_TEMPORAL2 ? 2 : 1; }
 Shape resolve_shape(int storage, const fdtd_tuning &t, int kind = 0, bool full_ch = false);
+void two_step_defaults(int nx, int ny, int nz, int storage, int sms, fdtd_tuning &t);   // host only
 Shape cavity_shape(const fdtd_ctx *c, int kind);
 int choose_zlen(long long cols, int nz, int grid, int zchunk, int prologue_planes);
 long long simulate_plan(const std::vector<int> &plan, long long cols, int G, int prologue);

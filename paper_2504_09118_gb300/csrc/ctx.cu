@@ -366,6 +366,16 @@ int fdtd_debug_resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]
     return FDTD_OK;
 }
 
+int fdtd_debug_two_step_shape(int nx, int ny, int nz, int storage, int sms, int *tile_y, int *stages) {
+    if (!tile_y || !stages || nx < 1 || ny < 1 || nz < 1 || sms < 1 || storage < FDTD_F32 || storage > FDTD_BF16)
+        return FDTD_ERR_ARG;
+    fdtd_tuning t{};
+    two_step_defaults(nx, ny, nz, storage, sms, t);
+    *tile_y = t.tile_y;
+    *stages = t.stages;
+    return FDTD_OK;
+}
+
 const char *fdtd_last_error(const fdtd_ctx *ctx) { return ctx ? ctx->err.c_str() : g_create_error.c_str(); }
 
 int fdtd_create(fdtd_ctx **out, int nx, int ny, int nz, double dt, double dx, const float *const ce[3],

@@ -242,40 +242,49 @@ std::vector<TileRec> assign_tiles(const std::vector<TileRec> &v, int G, int prol
     return out;
 }
 
-// Launch shape of a cavity's kernel of this kind.  The two-step kernel (one row per warp) picks the tile height
-// the tuning leaves open from the work split: the plan's makespan in plane-times, times the time a plane takes
-// with that height.  Measured per plane (us; 512^3, 256^3, 200 x 131 x 120): FP32 0.63, 0.62, 0.66 with 8 rows,
-// 0.89, 0.85, 0.87 with 12 and 1.23, 1.13, 1.17 with 16; 16-bit 0.57-0.60, 0.73-0.76, 0.92-0.95.  Taller tiles
-// recompute less halo but cut the cavity into fewer, larger pieces: per step, 16 against 12 rows, 200 x 131 x
-// 120 FP32 21.2 against 19.4 us, 384^3 262 against 246 us, 256^3 84.1 against 85.1 us, 512^3 608 against 593 us.
-// Ring depth left open, FP32: 16 rows 5 slots, 12 rows 6, the deepest that fit, but one less from kDeepRingCells
-// cells on, where the deeper ring makes the CTAs read more halo from DRAM (512^3: 4.07 against 3.61 GB a launch)
-// and run up to 40 % slower: 512^3 694 against 608 us (16 rows), 727 against 593 us (12); 448^3 447 against 411 and
-// 430 against 393 us; 512 x 512 x 256 (6.7e7 cells) still 288 against 301 and 284 against 293 us.
-Shape cavity_shape(const fdtd_ctx *c, int kind) {
-    constexpr long long kDeepRingCells = 75000000;
-    fdtd_tuning t = c->tuning;
-    if (kind == 1 && two_step_rows(t) == 1) {
-        const bool f32 = c->storage == FDTD_F32;
-        const long long cells = (long long)c->nx * c->ny * c->nz;
-        if (t.tile_y != 8 && t.tile_y != 12 && t.tile_y != 16) {
-            const double plane_us[3] = {f32 ? 0.62 : 0.58, f32 ? (cells < kDeepRingCells ? 0.86 : 0.89) : 0.75,
-                                        f32 ? (cells < kDeepRingCells ? 1.14 : 1.23) : 0.935};
-            const int tw = fused2_tile_w(c->storage);
-            double best = -1.0;
-            for (int q = 0; q < 3; ++q) {
-                const int ty = 8 + 4 * q;
-                const long long cols = (long long)((c->nx + tw - 1) / tw) * ((c->ny + ty - 1) / ty);
-                const int G = (int)std::min<long long>(num_sms(), cols * c->nz);
-                const double us = plane_us[q] * simulate_plan(plan_chunks(cols, c->nz, G, 3, t.zchunk), cols, G, 3);
-                if (best < 0 || us < best) {
-                    best = us;
-                    t.tile_y = ty;
-                }
+// What the two-step kernel (one row per warp) takes where the tuning leaves the tile height or the ring depth open.
+// Height: the plan's makespan in plane-times, times what a plane takes with that height, in relation to each other.
+// Taller tiles recompute less halo but cut the cavity into fewer, larger pieces: per step, 16 against 12 rows, 200 x 131 x
+// 120 FP32 19.7 against 19.0 us, 256^3 79.7 against 83.9, 474 x 184 x 230 87.3 against 94.6, 512^3 600 against 593.
+// A launch is 2-3 us and 0.65, 0.87 and 1.11 us a plane (FP32, 8, 12 and 16 rows; 16-bit 0.58, 0.73, 0.91), which
+// varies by 4 % with the shape, so the factors are those whose choice came out best: over 97 FP32 cavities of 4e5 to
+// 7.2e7 cells 0.3 % behind the best of the three heights (with 0.62 and 0.86 in place of 0.66 and 0.89: 1.7 %, and up to
+// 27 % slower than 16 rows), over 95 with 16-bit storage 0.2 %.
+// Ring depth, FP32: the deepest that fits (16 rows 5 slots, 12 rows 6, 8 rows 8) until the CTAs, further apart in z, no
+// longer find each other's halo in L2: 512^3 with 16 rows and 5 slots reads 4.07 GB a launch, with 4 slots 3.61.  How much
+// depends on the shape; the shallower rings take 4.2-5.0 ps per cell and step everywhere, the deeper 3.9-6.0 (24 cavities
+// of 5.7e7 to 1.7e8 cells).  16 rows, 5 against 4 slots: 512^3 5.00 / 4.46, 448^3 4.84 / 4.56, 542 x 560 x 491 5.96 / 4.69,
+// 410 x 410 x 535 4.22 / 4.41, 512 x 512 x 256 4.23 / 4.52: 4 from kDeepRing16 cells on.  12 rows, 6 against 5: 512^3
+// 5.40 / 4.43, 323 x 263 x 844 5.39 / 4.72, 271 x 704 x 340 5.18 / 4.61, 717 x 302 x 785 4.11 / 4.24, 384^3 4.40 / 4.45:
+// 5 from kDeepRing12 cells on.  12 rows and 5 slots are 7.8 % slower than 16 and 5 at worst (399 x 762 x 457), 28 % faster
+// at best, 6 % on average.
+void two_step_defaults(int nx, int ny, int nz, int storage, int sms, fdtd_tuning &t) {
+    constexpr long long kDeepRing16 = 75000000, kDeepRing12 = 50000000;
+    const bool f32 = storage == FDTD_F32;
+    const long long cells = (long long)nx * ny * nz;
+    if (t.tile_y != 8 && t.tile_y != 12 && t.tile_y != 16) {
+        const double plane_us[3] = {f32 ? 0.66 : 0.58, f32 ? 0.89 : 0.75, f32 ? (cells < kDeepRing16 ? 1.14 : 1.23) : 0.935};
+        const int tw = fused2_tile_w(storage);
+        double best = -1.0;
+        for (int q = 0; q < 3; ++q) {
+            const int ty = 8 + 4 * q;
+            const long long cols = (long long)((nx + tw - 1) / tw) * ((ny + ty - 1) / ty);
+            const int G = (int)std::min<long long>(sms, cols * nz);
+            const double us = plane_us[q] * simulate_plan(plan_chunks(cols, nz, G, 3, t.zchunk), cols, G, 3);
+            if (best < 0 || us < best) {
+                best = us;
+                t.tile_y = ty;
             }
         }
-        if (t.stages == 0 && f32 && cells >= kDeepRingCells) t.stages = t.tile_y == 16 ? 4 : t.tile_y == 12 ? 5 : 6;
     }
+    if (t.stages == 0 && f32 && t.tile_y == 12 && cells >= kDeepRing12) t.stages = 5;
+    if (t.stages == 0 && f32 && cells >= kDeepRing16) t.stages = t.tile_y == 16 ? 4 : 6;
+}
+
+// Launch shape of a cavity's kernel of this kind.
+Shape cavity_shape(const fdtd_ctx *c, int kind) {
+    fdtd_tuning t = c->tuning;
+    if (kind == 1 && two_step_rows(t) == 1) two_step_defaults(c->nx, c->ny, c->nz, c->storage, num_sms(), t);
     return resolve_shape(c->storage, t, kind, !c->ch_uniform);
 }
 

@@ -58,3 +58,28 @@ def test_small_cavities_leave_room_for_other_launches():
     for dims, most in (((16, 16, 16), SMS // 8), ((24, 20, 17), SMS // 8), ((32, 32, 32), SMS // 4)):
         px, py, pz = B.fdtd_debug_resident_split(*dims, SMS)
         assert px * py * pz <= most
+
+
+# cavities where a height is ahead of both others by 4 % or more (us per step with 8, 12 and 16 rows, FP32)
+HEIGHTS = [((474, 184, 230), 16), ((160, 150, 140), 16), ((482, 195, 147), 16), ((305, 311, 274), 16), ((230, 850, 340), 16),
+           ((172, 143, 50), 12), ((243, 69, 75), 12), ((164, 499, 124), 12), ((459, 227, 270), 12), ((55, 31, 32), 8)]
+
+
+@pytest.mark.parametrize("dims,rows", HEIGHTS)
+def test_two_step_height_is_the_measured_best(dims, rows):
+    assert B.fdtd_debug_two_step_shape(*dims, B.FDTD_F32, SMS)[0] == rows
+
+
+def test_two_step_ring_depth_by_size():
+    """Both sides of the sizes from which FP32 rings are shallower; 16-bit rings always fill the shared memory."""
+    shape = lambda dims, storage=B.FDTD_F32: B.fdtd_debug_two_step_shape(*dims, storage, SMS)
+    assert shape((512, 512, 512)) == (12, 5)
+    assert shape((323, 263, 844)) == (12, 5)          # 7.2e7 cells
+    assert shape((459, 227, 270)) == (12, 0)          # 2.8e7
+    assert shape((512, 512, 256)) == (16, 0)          # 6.7e7
+    for dims in ((512, 512, 512), (323, 263, 844), (459, 227, 270)):
+        for storage in (B.FDTD_F16, B.FDTD_BF16):
+            assert shape(dims, storage)[1] == 0
+    for storage in (B.FDTD_F32, B.FDTD_BF16):         # one cell to the largest axes
+        for dims in ((1, 1, 1), (1, 1, 32768), (32768, 1, 1), (1, 32768, 3), (61, 17, 5)):
+            assert shape(dims, storage)[0] in (8, 12, 16)
