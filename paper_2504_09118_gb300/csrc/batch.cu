@@ -341,7 +341,7 @@ static int batch_launch(fdtd_batch *b, int parity, int nsteps) {
     L.grid = b->grid;
     L.launch_steps = nsteps;
     L.rows_per_warp = s.rows_per_warp;
-    L.overlap = b->cells < kOverlapCells;
+    L.overlap = b->cells < kOverlapCellsBatch;
     L.coef_class = b->steady ? COEF_CLASS_ANY_STEADY : COEF_CLASS_ANY;
     cudaError_t e = kind == 0   ? launch_fused_step(b->storage, L, b->stream)
                     : kind == 1 ? launch_fused2_step(b->storage, L, b->stream)

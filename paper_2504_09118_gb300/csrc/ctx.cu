@@ -208,7 +208,7 @@ int launch_one(fdtd_ctx *c, int parity, int inject_us, int kind) {
     L.inject_timeout_us = inject_us;
     L.first = tl.first;
     L.rows_per_warp = s.rows_per_warp;
-    L.overlap = (long long)c->nx * c->ny * c->nz < kOverlapCells;
+    L.overlap = (long long)c->nx * c->ny * c->nz < (c->storage == FDTD_F32 ? kOverlapCells32 : kOverlapCells16);
     L.coef_class = coef_class_of(c->coef_mode, c->ch_uniform, kind == 1 && c->id_pec);
     if (kind == 0)
         CK(c, launch_fused_step(c->storage, L, c->stream));

@@ -61,9 +61,13 @@ template <typename Kernel> inline cudaError_t allow_all_smem(Kernel kern, int st
 // before it touches the fields).  Back to back, a tiled launch otherwise pays its launch latency, barrier set-up and
 // first ring fill after the slowest CTA of the launch before it: per launch 2-4 us of 30-40 (200 x 131 x 120 BF16: a
 // 64-step pass 1.44 -> 1.34 ms; 160 x 150 x 140 per-position 1.49 -> 1.39 ms).  CTAs started that way land on the SMs
-// in the order these fall free, which costs long launches more than it saves (512^3 FP32: 122.4 -> 124.8 ms for 100
-// launches), so launches over kOverlapCells cells start after the previous one.
-constexpr long long kOverlapCells = 30000000;
+// in the order these fall free, which moves neighbouring tiles apart and costs large FP32 cavities halo reads.  Two-step
+// kernel, us a step without and with overlap, FP32: 211 x 198 x 368 (1.5e7 cells) 79.3 / 77.8, 256^3 81.2 / 79.7,
+// 234 x 379 x 230 (2.0e7) 96.2 / 100.0, 115 x 354 x 521 (2.1e7) 108.0 / 109.6, 247 x 328 x 271 (2.2e7) 110.5 / 109.1,
+// 288^3 (2.4e7) 103.5 / 102.0, 320^3 145.7 / 145.0, 384^3 248.2 / 248.9, 512^3 596 / 600; BF16: 256^3 69.9 / 68.4, 288^3
+// 85.0 / 83.1, 384^3 204.7 / 202.8, 512^3 459 / 460.  So FP32 launches overlap below 2e7 cells, where all gain, and 16-bit
+// ones below 3e7 (a batch: its running members' cells).
+constexpr long long kOverlapCells32 = 20000000, kOverlapCells16 = 30000000, kOverlapCellsBatch = 30000000;
 template <typename Kernel, typename Params>
 inline cudaError_t launch_overlapped(Kernel kern, int grid, int threads, int smem, cudaStream_t s, const Params &p,
                                      bool overlap) {
