@@ -77,8 +77,8 @@ enum fdtd_kernel {
                                 on chip, many steps per launch (FP32: bit for bit the other kernels' results;
                                 16-bit storage is rounded once per launch).  Else TEMPORAL where it applies
                                 (second order, per-position coefficient arrays included), else FUSED, else
-                                SIMPLE (fourth order with per-position coefficient arrays); fdtd_autotune picks
-                                among the tiled kernels by timing */
+                                SIMPLE (fourth order with per-position coefficient arrays); fdtd_autotune
+                                times it against the tiled kernels in fixed shapes */
     FDTD_KERNEL_SIMPLE = 1,  /* two launches per step (H, then E), one thread per cell; unfused baseline */
     FDTD_KERNEL_FUSED = 2,   /* one TMA-pipelined launch per step: H then E fused in a z-march */
     FDTD_KERNEL_TEMPORAL = 3, /* two steps per launch (temporal blocking); an odd count ends with one FUSED step.
@@ -232,7 +232,7 @@ FDTD_API int fdtd_set_order(fdtd_ctx *ctx, int order);
 FDTD_API int fdtd_get_order(const fdtd_ctx *ctx);
 
 /* fdtd_autotune - choose the step kernel and launch shape by timing candidates on this
- * context's own state: the one-step kernel with 4, 8, 16-row tiles, the two-step kernel with
+ * context's own state: AUTO with an open launch shape, the one-step kernel with 4, 8, 16-row tiles, the two-step kernel with
  * 8, 12, 16-row tiles and 4 or 6 ring slots, the three-step kernel with 8, 10, 12-row tiles, and the
  * two-step kernel with two rows per warp with 12 and 16-row tiles (graphs on).  Each candidate runs trial_steps steps
  * (rounded up to a multiple of 16; <= 0: 16) after one untimed run of the same length, timed
@@ -240,8 +240,8 @@ FDTD_API int fdtd_get_order(const fdtd_ctx *ctx);
  * of the active arrays, freed before return) and restored afterwards, so the state and
  * fdtd_steps_done are unchanged.  The choice is kept per (nx, ny, nz, storage, coefficient
  * kind, spatial order) for the life of the process: a later call for the same shape applies it
- * without trials.  Contexts with per-position coefficient arrays are not timed and get SIMPLE (AUTO's
- * two-step kernel is faster on them: do not autotune those); with
+ * without trials.  Contexts with per-position coefficient arrays have one shape, are not timed and get AUTO
+ * (with order 4 SIMPLE); with
  * order 4 the candidates are the fused fourth-order kernel with 4, 8, 12, 16-row tiles and the
  * deepest ring that fits or 4 slots.  out
  * (may be NULL) receives the chosen tuning, ms_per_step (may be NULL) its time per step.
@@ -328,7 +328,7 @@ FDTD_API int fdtd_batch_step(fdtd_batch *b, int nsteps);
 FDTD_API int fdtd_batch_set_tuning(fdtd_batch *b, const fdtd_tuning *t);
 
 /* fdtd_batch_autotune - fdtd_autotune for a batch over its current members: the one-step kernel
- * with 4, 8, 16-row tiles and the two-step kernels with 8, 12, 16-row tiles (two rows per warp:
+ * with 4, 8, 16-row tiles, the two-step kernel with an open shape and with 8, 12, 16-row tiles (two rows per warp:
  * 12, 16), each timed over
  * trial_steps batch steps (rounded up to a multiple of 16; <= 0: 16) after an untimed run.
  * Members' fields, step counts and the batch clock are restored afterwards.  Not cached (the

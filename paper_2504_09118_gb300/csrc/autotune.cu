@@ -12,6 +12,8 @@ std::vector<fdtd_tuning> tune_candidates(bool batch, int order) {
             for (int st : {0, 4}) v.push_back(fdtd_tuning{FDTD_KERNEL_FUSED, ty, 0, 0, st, 1});
         return v;
     }
+    // what runs untuned: small single cavities on chip, else the two-step kernel in its own choice of shape
+    v.push_back(fdtd_tuning{batch ? FDTD_KERNEL_TEMPORAL : FDTD_KERNEL_AUTO, 0, 0, 0, 0, 1});
     for (int ty : {4, 8, 16}) v.push_back(fdtd_tuning{FDTD_KERNEL_FUSED, ty, 0, 0, 4, 1});
     for (int ty : {8, 12, 16})
         for (int st : {4, 6}) {
@@ -53,12 +55,14 @@ int fdtd_autotune(fdtd_ctx *c, int trial_steps, fdtd_tuning *out, double *ms_per
         if (ms_per_step) *ms_per_step = ms;
         return FDTD_OK;
     };
-    if (c->coef_mode == COEF_FULL) {   // per-position coefficient arrays: only the unfused kernel applies
-        fdtd_tuning t{FDTD_KERNEL_SIMPLE, 0, 0, 0, 0, c->tuning.use_graph};
+    if (c->coef_mode == COEF_FULL) {   // per-position coefficient arrays: the two-step kernel in its one shape, or unfused
+        fdtd_tuning t{c->order == 4 ? FDTD_KERNEL_SIMPLE : FDTD_KERNEL_AUTO, 0, 0, 0, 0, c->tuning.use_graph};
         if (int rc = fdtd_set_tuning(c, &t)) return rc;
         return report(t, -1.0);
     }
-    const auto key = std::make_tuple(c->nx, c->ny, c->nz, c->storage, c->coef_mode, c->ch_uniform, c->order);
+    // (cavities with more materials than the PEC coding takes run other instances, and never on chip)
+    const auto key = std::make_tuple(c->nx, c->ny, c->nz, c->storage, 2 * c->coef_mode + (c->id_pec ? 1 : 0),
+                                     c->ch_uniform, c->order);
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune_cache.find(key);

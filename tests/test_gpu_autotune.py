@@ -1,5 +1,6 @@
 """Autotuning (fdtd_autotune, fdtd_batch_autotune): the state is untouched and the pick is a valid shape.
 
+The candidates of a single cavity include its untuned state (kernel 0), so tuning never leaves it slower than no tuning.
 With FP32 storage every candidate produces bit-identical fields (same operation sequence per value),
 so a tuned run must equal an untuned run bit for bit.
 """
@@ -24,8 +25,8 @@ def test_autotune_keeps_state_and_result():
         cav.step(3)
         before = cav.get_fields()
         tuning, ms = cav.autotune(16)
-        assert tuning["kernel"] in (2, 3, 4, 5) and ms > 0
-        assert tuning["tile_y"] in {2: (4, 8, 16), 3: (8, 12, 16), 4: (12, 16), 5: (8, 10, 12)}[tuning["kernel"]]
+        assert tuning["kernel"] in (0, 2, 3, 4, 5) and ms > 0
+        assert tuning["tile_y"] in {0: (0,), 2: (4, 8, 16), 3: (8, 12, 16), 4: (12, 16), 5: (8, 10, 12)}[tuning["kernel"]]
         assert cav.steps_done == 3
         for x, y in zip(cav.get_fields(), before):
             assert np.array_equal(x, y)
@@ -41,16 +42,41 @@ def test_autotune_keeps_state_and_result():
             assert np.array_equal(x, y)
 
 
-def test_autotune_full_coefficients_keeps_unfused_kernel():
+@pytest.mark.parametrize("order,kernel", [(2, 0), (4, 1)])
+def test_autotune_full_coefficients(order, kernel):
+    """Per-position coefficients keep AUTO (the two-step kernel that streams them; one shape, nothing to time), the
+    fourth order the unfused kernel."""
     from paper_2504_09118_gb300 import Cavity
     dims = (12, 10, 9)
     rng = np.random.default_rng(2)
     sh = (dims[2] + 1, dims[1] + 1, dims[0] + 1)
-    ce = [(DT * rng.uniform(0.5, 1.0, sh)).astype(np.float32) for _ in range(3)]
-    with Cavity(*dims, DT, 1.0, ce, None) as cav:
-        cav.set_fields(ci.random_fields(1, *dims))
-        tuning, _ = cav.autotune()
-        assert tuning["kernel"] == 1
+    ce = [(0.5 * DT * rng.uniform(0.5, 1.0, sh)).astype(np.float32) for _ in range(3)]
+    f = ci.random_fields(1, *dims)
+    out = []
+    for tune in (False, True):
+        with Cavity(*dims, DT, 1.0, ce, None, order=order) as cav:
+            cav.set_fields(f)
+            if tune:
+                tuning, _ = cav.autotune()
+                assert tuning["kernel"] == kernel
+            cav.step(7)
+            out.append(cav.get_fields())
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+
+
+def test_autotune_never_leaves_a_small_cavity_off_chip():
+    """A cavity of the on-chip kernel's size steps about twice as fast on chip as in any tiled launch."""
+    from paper_2504_09118_gb300 import Cavity
+    dims = (64, 64, 64)
+    with Cavity(*dims, DT) as cav:
+        cav.set_fields(ci.random_fields(5, *dims))
+        cav.step(5)
+        before = cav.get_fields()
+        tuning, ms = cav.autotune(64)
+        assert tuning["kernel"] == 0 and ms > 0 and cav.steps_done == 5
+        for x, y in zip(cav.get_fields(), before):
+            assert np.array_equal(x, y)
 
 
 def test_batch_autotune_keeps_members():
