@@ -439,8 +439,9 @@ FDTD_API double fdtd_storage_scale_of(double maxabs);
  * Diagnostics
  * ------------------------------------------------------------------------ */
 
-/* fdtd_debug_inject_timeout - make the next fused step's first TMA stage never
- * be issued so that its bounded wait runs out after about limit_us microseconds;
+/* fdtd_debug_inject_timeout - make a wait of the next step call's first launch run out after about limit_us
+ * microseconds: on chip (AUTO, a small cavity of more than one box) one CTA waits for neighbour values that never come,
+ * else one fused step's first TMA stage is never issued;
  * the step then returns FDTD_ERR_TIMEOUT at the next synchronising call and the
  * context stays usable (its fields are undefined until the next set_fields).
  * Fault injection on the host side of a wait: no GPU fault is involved. */

@@ -936,9 +936,10 @@ static bool use_resident(fdtd_ctx *c, int nsteps) {
     return c->resident > 0;
 }
 
-// n steps on chip.  FDTD_OK with *done = false (nothing enqueued) when the device cannot run the launch or there
+// n steps on chip; inject_us > 0: with a wait that runs out after about that many microseconds (fdtd_debug_inject_timeout).
+// FDTD_OK with *done = false (nothing enqueued) when the device cannot run the launch or there
 // is no room for its buffers: the caller then takes the tiled kernels.
-static int step_resident(fdtd_ctx *c, int n, bool *done) {
+static int step_resident(fdtd_ctx *c, int n, int inject_us, bool *done) {
     *done = false;
     const int *parts = c->resident_parts;
     const size_t words = resident_word_bytes(c->nz, parts);
@@ -985,6 +986,7 @@ static int step_resident(fdtd_ctx *c, int n, bool *done) {
     P.words = c->d_resident;
     P.epoch = reinterpret_cast<unsigned *>(static_cast<char *>(c->d_resident) + words);
     P.status = c->d_status;
+    P.lose_polls = inject_us;   // a poll round takes about a microsecond
     if (extras_on(c)) P.X = make_extras(c);
     c->launched = true;
     const cudaError_t e = launch_resident(P, c->stream);
@@ -1015,15 +1017,17 @@ int fdtd_step(fdtd_ctx *c, int nsteps) {
     const bool temporal = (use_temporal(c) && !extras) || full2;
     const int k1 = one_step_kind(c);
     int left = nsteps;
-    if (c->inject_us <= 0)
-        while (use_resident(c, left)) {
-            const int launches = (left + kResidentMaxSteps - 1) / kResidentMaxSteps;
-            const int n = (left + launches - 1) / launches;   // equal shares: no short last launch
-            bool done = false;
-            if (int rc = step_resident(c, n, &done)) return rc;
-            if (!done) break;
-            left -= n;
-        }
+    while (use_resident(c, left)) {
+        // a wait to be lost needs a second box to wait for: a single one leaves it to the tiled launch below
+        if (c->inject_us > 0 && c->resident_parts[0] * c->resident_parts[1] * c->resident_parts[2] == 1) break;
+        const int launches = (left + kResidentMaxSteps - 1) / kResidentMaxSteps;
+        const int n = (left + launches - 1) / launches;   // equal shares: no short last launch
+        bool done = false;
+        if (int rc = step_resident(c, n, c->inject_us, &done)) return rc;
+        if (!done) break;
+        c->inject_us = 0;
+        left -= n;
+    }
     if (left == 0) return FDTD_OK;
     if (fused)
         if (int rc = build_tiles(c, k1)) return rc;

@@ -27,8 +27,8 @@
 // taken theirs of step s, because they send after a barrier behind their loads, and neighbours read each
 // other in pairs.  Tags go on from launch to launch (a device counter that the last CTA to read it advances),
 // so buffers are never cleared.
-// All CTAs run at once (cooperative launch).  Waits are bounded in wall time; the first to run out latches
-// STATUS_TIMEOUT, which every wait looks at, so that all CTAs leave.
+// All CTAs run at once (cooperative launch).  Waits are bounded in poll rounds (kPolls); the first to run out
+// latches STATUS_TIMEOUT, which every wait looks at, so that all CTAs leave without a result.
 #include <algorithm>
 
 #include "fused_common.cuh"
@@ -95,12 +95,12 @@ __device__ __forceinline__ void st_word(WordMem *p, float a, float b, float c, u
                  : "memory");
 }
 // Polls the wanted words (bit c of want) until every tag is the step's: all missing words of a round are
-// loaded together.  A round is an L2 round trip, so kPolls of them take over a second; a timer read per round
-// would cost as much as the round.
+// loaded together.  Gives up after `polls` rounds, or when another CTA has, and looks at either every 256.  A round is
+// an L2 round trip, about a microsecond, so kPolls are some seconds; a timer read per round would cost as much.
 constexpr int kPolls = 1 << 22;
 template <int N>
-__device__ __forceinline__ void wait_words(const WordMem *const *p, Word *v, unsigned want, unsigned tag, int *status,
-                                           int *abort) {
+__device__ __forceinline__ void wait_words(const WordMem *const *p, Word *v, unsigned want, unsigned tag, int polls,
+                                           int *status, int *abort) {
     for (int n = 1;; ++n) {
         bool miss = false;
 #pragma unroll
@@ -111,7 +111,7 @@ __device__ __forceinline__ void wait_words(const WordMem *const *p, Word *v, uns
             }
         if (!miss) return;
         if ((n & 255) == 0) {
-            if (n >= kPolls) atomicOr(status, STATUS_TIMEOUT);
+            if (n >= polls) atomicOr(status, STATUS_TIMEOUT);
             if (*(volatile int *)status != 0) {   // a wait ran out, here or in another CTA
                 *(volatile int *)abort = 1;
                 return;
@@ -188,6 +188,15 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentParams P)
     }
     __syncthreads();
     const unsigned tag0 = s_tag;
+    if (P.lose_polls > 0 && b == 0) {   // diagnostic: CTA 0 waits for a tag that nobody sends, its neighbours then for it
+        if (t == 0) {
+            const WordMem *const p[1] = {static_cast<const WordMem *>(P.words)};
+            Word v[1] = {{0, 0}};
+            wait_words<1>(p, v, 1u, tag0 ^ (1u << 31), P.lose_polls, P.status, &s_abort);
+        }
+        __syncthreads();
+        if (s_abort) return;
+    }
     unsigned src_mask = 0;   // planes of this thread's column that hold a current
     if (X.nsrc | X.nprobe) {
         // position of an active-array offset relative to the box
@@ -480,7 +489,7 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentParams P)
 #pragma unroll
             for (int c = 0; c < 7; ++c)
                 if ((want >> c) & 1u) v[c] = ld_word(p[c]);
-            wait_words<7>(p, v, want, tag, P.status, &s_abort);
+            wait_words<7>(p, v, want, tag, kPolls, P.status, &s_abort);
             if (zl) {
                 float *q = se + L::e(i, j, -1);
                 q[0] = v[0].a();

@@ -149,6 +149,7 @@ struct ResidentParams {
     void *words;               // surface buffers of every box, two copies (resident_word_bytes, zero at first)
     unsigned *epoch;           // step tag the next launch starts from, and a count of CTAs (both 0 at first)
     int *status;
+    int lose_polls;            // diagnostic, > 0: a wait of CTA 0 runs out after this many poll rounds
     ExtrasParams X;            // currents and probes (nsrc = nprobe = 0: none); advances X.clock
 };
 bool resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]);

@@ -111,3 +111,29 @@ def test_currents_and_probes_equal_the_per_step_launches(coef, dims):
     np.testing.assert_array_equal(res[0][1], res[1][1])
     for a, b in zip(res[0][0], res[1][0]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("dims", [(32, 16, 3), (40, 33, 21), (128, 96, 80), (16, 16, 2)])
+def test_a_wait_that_runs_out_ends_the_launch_and_the_context_recovers(dims):
+    """One CTA waits for words that never come: the launch ends with a latched timeout, also for the CTAs that wait for
+    that one; after a reload the step tags and surface buffers serve the next launches bit for bit.  (One box alone waits
+    for nothing: its timeout is that of a tiled launch.)"""
+    from paper_2504_09118_gb300 import Cavity, FdtdError, binding
+    ce, ch = _coef("spheres", dims)
+    f = ci.random_fields(15, *dims)
+    want, _ = _run(dims, (ce, ch), f, (9, 600))
+    with Cavity(*dims, DT, 1.0, ce, ch) as cav:
+        for before in (0, 7):
+            cav.set_fields(f)
+            cav.step(before)
+            binding.fdtd_debug_inject_timeout(cav.handle, 2000)
+            cav.step(300)     # two launches on chip: the second starts with the status latched
+            with pytest.raises(FdtdError) as e:
+                cav.sync()
+            assert e.value.code == binding.FDTD_ERR_TIMEOUT
+            cav.sync()        # reported once
+            cav.set_fields(f)
+            cav.step(9)
+            cav.step(600)
+            for a, b in zip(cav.get_fields(), want):
+                np.testing.assert_array_equal(a, b)
