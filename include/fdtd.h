@@ -496,6 +496,10 @@ FDTD_API int fdtd_debug_exchange_route(int lo_device, int hi_device, int current
  * cavity into with max_ctas CTAs at most (0, 0, 0: the cavity does not fit). */
 FDTD_API int fdtd_debug_resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]);
 
+/* fdtd_debug_halo_rows - host only: rows that a fused kernel's boxes hold beyond its tile's.  kind 0: one step, 1: two
+ * steps, 2: one fourth-order step, 3: three steps, 4: two steps with per-position coefficients (their boxes too). */
+FDTD_API int fdtd_debug_halo_rows(int kind);
+
 /* fdtd_debug_two_step_shape - host only: the tile height and ring depth (0: the deepest that fits) that the two-step
  * kernel takes for a cavity on a GPU of `sms` SMs where fdtd_tuning leaves both open. */
 FDTD_API int fdtd_debug_two_step_shape(int nx, int ny, int nz, int storage, int sms, int *tile_y, int *stages);

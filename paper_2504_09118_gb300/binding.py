@@ -35,6 +35,7 @@ EXPORTS = (
     "fdtd_get_probes", "fdtd_set_order", "fdtd_get_order", "fdtd_batch_retune", "fdtd_prefetch_fields",
     "fdtd_set_fields_prefetched", "fdtd_debug_fail_alloc", "fdtd_debug_tile_plan", "fdtd_debug_pec_code",
     "fdtd_debug_pec_table", "fdtd_debug_exchange_route", "fdtd_debug_resident_split", "fdtd_debug_two_step_shape",
+    "fdtd_debug_halo_rows",
     "fdtd_create_slab", "fdtd_slab_info", "fdtd_slab_halo_bytes", "fdtd_slab_export", "fdtd_slab_import",
     "fdtd_slab_exchange", "fdtd_slab_energy", "fdtd_slab_divergence_sq", "fdtd_set_storage_scales",
     "fdtd_storage_scale_of",
@@ -119,6 +120,7 @@ def lib() -> ctypes.CDLL:
             L.fdtd_debug_pec_table.argtypes = [vp, i, vp]
             L.fdtd_debug_exchange_route.argtypes = [i, i, i, i]
             L.fdtd_debug_resident_split.argtypes = [i, i, i, i, vp]
+            L.fdtd_debug_halo_rows.argtypes = [i]
             L.fdtd_debug_two_step_shape.argtypes = [i, i, i, i, i, ctypes.POINTER(i), ctypes.POINTER(i)]
             L.fdtd_set_fields_prefetched.argtypes = [vp]
             L.fdtd_batch_retune.argtypes = [vp, i, ctypes.POINTER(fdtd_tuning), ctypes.POINTER(d),
@@ -383,6 +385,14 @@ def fdtd_debug_resident_split(nx: int, ny: int, nz: int, max_ctas: int) -> tuple
     if rc != FDTD_OK:
         raise FdtdError(rc, "fdtd_debug_resident_split: invalid arguments")
     return tuple(parts) if parts[0] else None
+
+
+def fdtd_debug_halo_rows(kind: int) -> int:
+    """Host-only: rows that a fused kernel's boxes hold beyond its tile's (kind 0..4, see fdtd.h)."""
+    rc = int(lib().fdtd_debug_halo_rows(int(kind)))
+    if rc < 0:
+        raise FdtdError(rc, "fdtd_debug_halo_rows: invalid kind")
+    return rc
 
 
 def fdtd_debug_two_step_shape(nx: int, ny: int, nz: int, storage: int, sms: int) -> tuple[int, int]:

@@ -236,6 +236,8 @@ int ensure_stage(fdtd_ctx *c);
 int ensure_stage2(fdtd_ctx *c);
 
 // ---- launch planning (plan.cu)
+// Rows that a kernel's boxes hold beyond its tile's (kinds as in Shape): twice the reach of the steps of a launch.
+constexpr int halo_rows(int kind) { return kind == 0 ? 2 : kind == 1 || kind == 4 ? 4 : 6; }
 // Rows per consumer warp of the two-step kernel a tuning selects.
 inline int two_step_rows(const fdtd_tuning &t) { return t.kernel == FDTD_KERNEL_TEMPORAL2 ? 2 : 1; }
 Shape resolve_shape(int storage, const fdtd_tuning &t, int kind = 0, bool full_ch = false);

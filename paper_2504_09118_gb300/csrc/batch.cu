@@ -210,7 +210,7 @@ static int batch_rebuild(fdtd_batch *b) {
     fdtd_tuning tuning = b->tuning;
     if (kind == 1 && two_step_rows(tuning) == 1 && tuning.tile_y != 8 && tuning.tile_y != 16) tuning.tile_y = 12;
     Shape s = resolve_shape(b->storage, tuning, kind);
-    const int box_y = s.tile_y + (kind == 0 ? 2 : kind == 1 ? 4 : 6);
+    const int box_y = s.tile_y + halo_rows(kind);
     const int G = num_sms() * s.ctas_per_sm;
     std::vector<TileRec> tiles;
     long long total_cols_planes = 0;

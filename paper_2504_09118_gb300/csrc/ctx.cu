@@ -366,6 +366,8 @@ int fdtd_debug_resident_split(int nx, int ny, int nz, int max_ctas, int parts[3]
     return FDTD_OK;
 }
 
+int fdtd_debug_halo_rows(int kind) { return kind < 0 || kind > 4 ? FDTD_ERR_ARG : halo_rows(kind); }
+
 int fdtd_debug_two_step_shape(int nx, int ny, int nz, int storage, int sms, int *tile_y, int *stages) {
     if (!tile_y || !stages || nx < 1 || ny < 1 || nz < 1 || sms < 1 || storage < FDTD_F32 || storage > FDTD_BF16)
         return FDTD_ERR_ARG;

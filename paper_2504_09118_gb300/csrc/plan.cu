@@ -292,8 +292,7 @@ int build_tiles(fdtd_ctx *c, int kind) {
     fdtd_ctx::TileList &tl = c->tl[kind];
     if (tl.ready) return FDTD_OK;
     const Shape s = cavity_shape(c, kind);
-    int rc = kind == 4 ? encode_maps(c, kind, s.tile_y + 4)
-                       : encode_maps(c, kind, s.tile_y + (kind == 0 ? 2 : kind == 1 ? 4 : 6));
+    const int rc = encode_maps(c, kind, s.tile_y + halo_rows(kind));
     if (rc) return rc;
     const int tw = kind == 1 || kind == 4 ? fused2_tile_w(c->storage) : kind == 3 ? fused3_tile_w() : kTileX;
     const long long cols = (long long)((c->nx + tw - 1) / tw) * ((c->ny + s.tile_y - 1) / s.tile_y);

@@ -5,22 +5,19 @@ the cell.  A fused kernel that advances s steps per launch loads a box of (tile 
 of s steps, so a stored value never needs an input outside its box:
 
   one-step kernel (Eq. 2)        s = 1, R = 1   box rows tile_y + 2
-  two-step kernel (Eq. 2 twice)  s = 2, R = 2   box rows tile_y + 4
+  two-step kernel (Eq. 2 twice)  s = 2, R = 2   box rows tile_y + 4 (with per-position coefficients: their boxes too)
   fourth-order kernel            s = 1, R = 3   box rows tile_y + 6
-  three-step kernel              s = 3, R = 3   box rows tile_y + 6 (the same branch as the fourth order)
+  three-step kernel              s = 3, R = 3   box rows tile_y + 6
 
 The reach is also tight (some output does depend on a cell R away), so none of the boxes could be
-smaller.  The box heights are read from the host code that encodes the tensor maps."""
-import os
-import re
-
+smaller.  The halo rows come from the library: the function that sizes the tensor maps."""
 import numpy as np
 import pytest
 
 import cavity_inputs as ci
 import oracle
+from paper_2504_09118_gb300 import binding as B
 
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 N = 20
 C = (10, 10, 10)   # perturbed cell (k, j, i), far from the walls at these step counts
 
@@ -50,13 +47,7 @@ def test_reach_of_the_schemes(order, steps, expected):
     assert reach(order, steps) == (expected,) * 3
 
 
-def test_box_heights_cover_the_reach_exactly():
-    src = open(os.path.join(ROOT, "paper_2504_09118_gb300", "csrc", "plan.cu")).read()
-    m = re.search(r"encode_maps\(c, kind, s\.tile_y \+ \(kind == 0 \? (\d+) : kind == 1 \? (\d+) : (\d+)\)\)", src)
-    assert m, "box-height expression not found in plan.cu"
-    one_step, two_step, fourth = (int(g) for g in m.groups())
-    assert one_step == 2 * reach(2, 1)[1]
-    assert two_step == 2 * reach(2, 2)[1]
-    assert fourth == 2 * reach(4, 1)[1]
-    # kind 3 (three steps per launch) takes the last branch too
-    assert fourth == 2 * reach(2, 3)[1]
+@pytest.mark.parametrize("kind,order,steps", [(0, 2, 1), (1, 2, 2), (2, 4, 1), (3, 2, 3), (4, 2, 2)],
+                         ids=["one step", "two steps", "fourth order", "three steps", "two steps, per-position"])
+def test_box_heights_cover_the_reach_exactly(kind, order, steps):
+    assert B.fdtd_debug_halo_rows(kind) == 2 * reach(order, steps)[1]
