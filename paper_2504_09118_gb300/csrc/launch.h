@@ -110,7 +110,6 @@ inline int coef_class_of(int coef_mode, int ch_uniform, bool pec_ids) {
 int fused_smem_bytes(int storage, int tile_y, int stages);
 cudaError_t fused_occupancy(int storage, int tile_y, int stages, int *ctas_per_sm);
 cudaError_t launch_fused_step(int storage, const FusedLaunch &L, cudaStream_t s);
-// *counter += 1 on the stream (advances a batch's device launch counter after each step).
 // Point currents and probes applied after a step (k_extras.cu).
 struct ExtrasParams {
     long long *clock;          // device: steps taken since fdtd_set_fields; advanced by the launch
