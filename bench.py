@@ -76,9 +76,9 @@ WORKLOADS = {
 # temporal-blocking kernel, 60 x 16-cell tiles (FP32), 4-slot TMA ring (what fits beside 16-row
 # planes), graphs of 8 launches.
 BENCH_TUNING = dict(kernel=3, tile_y=16, stages=4, zchunk=0, ctas_per_sm=0, use_graph=1)
-# Batches of the serving loop: two-step launches, 16-row tiles (what fdtd_batch_autotune picks for the
-# batch workload, and measured best on the serving stream; the mix changes every chunk, so it is fixed
-# rather than re-tuned).
+# Batches of the serving loop: two-step launches, 16-row tiles, fixed rather than re-tuned since the mix changes every
+# chunk (fdtd_batch_autotune picks the open shape, 12 rows with steady bodies, for the batch workload; not measured on
+# the serving stream).
 SERVE_TUNING = dict(kernel=3, tile_y=16, stages=4)
 STEPS_PER_LAUNCH = {1: 0.5, 2: 1, 3: 2, 4: 2, 5: 3}   # leapfrog steps per launch of each kernel kind (SIMPLE: H and E launches)
 DOMINANT_KERNEL = {1: "simple_h_kernel/simple_e_kernel", 2: "fused_step_kernel", 3: "fused2_step_kernel",
